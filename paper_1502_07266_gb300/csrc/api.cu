@@ -175,6 +175,7 @@ void free_ctx(helm_ctx* h) {
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete[] h->prob_h;
+    delete[] static_cast<AxisWin*>(h->win_h);
     delete h;
 }
 
@@ -365,6 +366,9 @@ int helm_setup(const float* c, double omega, int n, int b, int d, const helm_opt
     h->dense = dense ? 1 : 0;
     h->prob_h = new Prob[prob.size()];
     memcpy(h->prob_h, prob.data(), sizeof(Prob) * prob.size());
+    AxisWin* wh = new AxisWin[B];
+    memcpy(wh, win.data(), sizeof(AxisWin) * B);
+    h->win_h = wh;
     cudaGetDevice(&h->device);
     cudaStream_t st = (cudaStream_t)stream;
     const size_t n3 = (size_t)N * N * N;

@@ -62,20 +62,9 @@ __device__ __forceinline__ void cfma(float2& acc, float2 a, float2 b) {
 
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
-// Exponent of the power-of-two scale that puts a largest magnitude f 2^ex
-// (f in [0.5, 1)) into [2^14, 2^15), clamped so that both the scale and its
-// inverse stay normal FP32 numbers: an almost-zero row or column (below about
-// 2^-105) is scaled by 2^120 only, its FP16 parts then losing digits that are
-// negligible next to the other rows and columns of the product.
-__host__ __device__ __forceinline__ int scale_exp(int ex) {
-    const int e = 15 - ex;
-    return e < -120 ? -120 : (e > 120 ? 120 : e);
-}
-
-// Bytes per K column of the main part of one stored tile: 64 complex rows in
-// FP32 (512), or 128 real rows of FP16 hi + lo (512) or hi only (256).  A tile
-// also carries xr extra complex rows in FP32 (8 bytes per row and K column).
-int tile_unit(int precision) { return precision == HELM_FP16 ? 256 : 512; }
+// Bytes per K column of the main part of one stored tile (FP32 form): 64 complex
+// rows.  A tile also carries xr extra complex rows (8 bytes per row and K column).
+constexpr int TILE_UNIT = 512;
 
 #include "dense_sched.h"
 
@@ -327,105 +316,43 @@ k_dense_G(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __restric
     }
 }
 
-// Real rows of an FP16 tile: the 64 complex rows' real parts and imaginary
-// parts, interleaved in groups of 16 so that both parts of a complex row land
-// in the same 32-lane quarter of the MMA accumulator (one warp reads both):
-// tile row rho = 32 (i / 16) + 16 part + i mod 16 for complex row i.
-__host__ __device__ __forceinline__ int tile_row(int i, int part) { return 32 * (i >> 4) + 16 * part + (i & 15); }
-__host__ __device__ __forceinline__ int tile_cplx(int rho) { return 16 * (rho >> 5) + (rho & 15); }
-__host__ __device__ __forceinline__ int tile_part(int rho) { return (rho >> 4) & 1; }
-
 // Pack one output tile (operator p, 64 complex rows) into the apply's format.
 struct PItem { int p, mt; };
 
-template <int FMT>
 __global__ void __launch_bounds__(256)
 k_dense_pack(const DProb* __restrict__ dp, const PItem* __restrict__ items, const float2* __restrict__ Gt,
-             const long long* __restrict__ goff, unsigned char* __restrict__ G, float* __restrict__ scale) {
-    __shared__ float s_sc[128];
+             const long long* __restrict__ goff, unsigned char* __restrict__ G) {
     __shared__ float2 stage[64][33];
     const PItem I = items[blockIdx.x];
     const DProb D = dp[I.p];
     const float2* src = Gt + goff[I.p];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x;
     const int n_in = D.n_in;
     const int row0 = I.mt * (64 + D.xr);             // first output row of the tile
-    if (FMT != HELM_FP32) {
-        // one power-of-two scale per real row: its largest |part| into [2^14, 2^15)
-        for (int rho = warp; rho < 128; rho += 8) {
-            const int o = row0 + tile_cplx(rho), part = tile_part(rho);
-            float mx = 0.f;
-            if (o < D.n_out)
-                for (int j = lane; j < n_in; j += 32) {
-                    const float2 v = src[(size_t)o * n_in + j];
-                    mx = fmaxf(mx, fabsf(part ? v.y : v.x));
-                }
-            for (int s = 16; s > 0; s >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
-            if (lane == 0) {
-                float sc = 1.f;
-                if (mx > 0.f) {
-                    int ex;
-                    frexpf(mx, &ex);
-                    sc = ldexpf(1.f, scale_exp(ex));
-                }
-                s_sc[rho] = sc;
-                scale[D.soff + (long long)I.mt * 128 + rho] = sc;
-            }
-        }
-        __syncthreads();
-    }
-    const int unit = (FMT == HELM_FP16) ? 256 : 512;
-    const int unit_x = unit + 8 * D.xr;
+    const int unit_x = TILE_UNIT + 8 * D.xr;
     for (int r = 0; r < HELM_DENSE_CS; ++r) {
         for (int c = 0; c < D.nkc; ++c) {
             const int kw = min(128, D.KR - 128 * c);
             const int jb = r * D.KR + 128 * c;
             unsigned char* tile = G + D.off + ((long long)(I.mt * HELM_DENSE_CS + r) * D.KR + 128 * c) * unit_x;
-            if (FMT == HELM_FP32) {
-                // [kw][64] complex: element (kj, row) at kj * 64 + row
-                float2* T = reinterpret_cast<float2*>(tile);
-                for (int k0 = 0; k0 < kw; k0 += 32) {
-                    __syncthreads();
-                    for (int e = tid; e < 64 * 32; e += 256) {
-                        const int row = e >> 5, kj = e & 31;
-                        const int o = row0 + row, j = jb + k0 + kj;
-                        stage[row][kj] = (row < 64 && o < D.n_out && j < n_in && k0 + kj < kw)
-                                             ? src[(size_t)o * n_in + j] : make_float2(0.f, 0.f);
-                    }
-                    __syncthreads();
-                    for (int e = tid; e < 64 * 32; e += 256) {
-                        const int kj = e >> 6, row = e & 63;
-                        if (k0 + kj < kw) T[(size_t)(k0 + kj) * 64 + row] = stage[row][kj];
-                    }
+            // [kw][64] complex: element (kj, row) at kj * 64 + row
+            float2* T = reinterpret_cast<float2*>(tile);
+            for (int k0 = 0; k0 < kw; k0 += 32) {
+                __syncthreads();
+                for (int e = tid; e < 64 * 32; e += 256) {
+                    const int row = e >> 5, kj = e & 31;
+                    const int o = row0 + row, j = jb + k0 + kj;
+                    stage[row][kj] = (row < 64 && o < D.n_out && j < n_in && k0 + kj < kw)
+                                         ? src[(size_t)o * n_in + j] : make_float2(0.f, 0.f);
                 }
-            } else {
-                // 128 real rows (real and imaginary parts in the tile_row order) x kw,
-                // FP16, K-major core-matrix layout; the lo tile follows the hi tile
-                const int sbo = (kw / 8) * 128;
-                for (int e = tid; e < 128 * (kw / 8); e += 256) {
-                    const int rho = e / (kw / 8), kg = e - rho * (kw / 8);
-                    const int o = row0 + tile_cplx(rho), part = tile_part(rho);
-                    const float sc = s_sc[rho];
-                    __align__(16) __half hi[8], lo[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int j = jb + 8 * kg + q;
-                        float v = 0.f;
-                        if (o < D.n_out && j < n_in) {
-                            const float2 z = src[(size_t)o * n_in + j];
-                            v = (part ? z.y : z.x) * sc;
-                        }
-                        hi[q] = __float2half_rn(v);
-                        lo[q] = __float2half_rn(v - __half2float(hi[q]));
-                    }
-                    const size_t pos = (size_t)(rho >> 3) * sbo + (size_t)kg * 128 + (rho & 7) * 16;
-                    *reinterpret_cast<uint4*>(tile + pos) = *reinterpret_cast<const uint4*>(hi);
-                    if (FMT == HELM_SPLIT_FP16)
-                        *reinterpret_cast<uint4*>(tile + (size_t)128 * kw * 2 + pos) = *reinterpret_cast<const uint4*>(lo);
+                __syncthreads();
+                for (int e = tid; e < 64 * 32; e += 256) {
+                    const int kj = e >> 6, row = e & 63;
+                    if (k0 + kj < kw) T[(size_t)(k0 + kj) * 64 + row] = stage[row][kj];
                 }
             }
-            // extra rows: complex FP32 [xr][kw] after the main part
-            float2* X = reinterpret_cast<float2*>(tile + (size_t)unit * kw);
+            // extra rows: [xr][kw] after the main part
+            float2* X = reinterpret_cast<float2*>(tile + (size_t)TILE_UNIT * kw);
             for (int e = tid; e < D.xr * kw; e += 256) {
                 const int x = e / kw, kj = e - x * kw;
                 const int o = row0 + 64 + x, j = jb + kj;
@@ -436,12 +363,9 @@ k_dense_pack(const DProb* __restrict__ dp, const PItem* __restrict__ items, cons
 }
 
 // Read one stored operator back as complex FP32 [n_out][n_in] (for tests).
-template <int FMT>
-__global__ void k_dense_unpack(DProb D, const unsigned char* __restrict__ G, const float* __restrict__ scale,
-                               float2* __restrict__ out) {
+__global__ void k_dense_unpack(DProb D, const unsigned char* __restrict__ G, float2* __restrict__ out) {
     const long long total = (long long)D.n_out * D.n_in;
-    const int unit = (FMT == HELM_FP16) ? 256 : 512;
-    const int unit_x = unit + 8 * D.xr, rows = 64 + D.xr;
+    const int unit_x = TILE_UNIT + 8 * D.xr, rows = 64 + D.xr;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
         const int o = (int)(e / D.n_in), j = (int)(e - (long long)o * D.n_in);
@@ -449,25 +373,8 @@ __global__ void k_dense_unpack(DProb D, const unsigned char* __restrict__ G, con
         const int r = j / D.KR, jr = j - r * D.KR, c = jr >> 7, kj = jr & 127;
         const int kw = min(128, D.KR - 128 * c);
         const unsigned char* tile = G + D.off + ((long long)(mt * HELM_DENSE_CS + r) * D.KR + 128 * c) * unit_x;
-        float2 v;
-        if (row >= 64) {
-            v = reinterpret_cast<const float2*>(tile + (size_t)unit * kw)[(size_t)(row - 64) * kw + kj];
-        } else if (FMT == HELM_FP32) {
-            v = reinterpret_cast<const float2*>(tile)[(size_t)kj * 64 + row];
-        } else {
-            const int sbo = (kw / 8) * 128;
-            float part[2];
-            for (int q = 0; q < 2; ++q) {
-                const int rho = tile_row(row, q);
-                const size_t pos = (size_t)(rho >> 3) * sbo + (size_t)(kj >> 3) * 128 + (rho & 7) * 16 + (kj & 7) * 2;
-                float x = __half2float(*reinterpret_cast<const __half*>(tile + pos));
-                if (FMT == HELM_SPLIT_FP16)
-                    x += __half2float(*reinterpret_cast<const __half*>(tile + (size_t)128 * kw * 2 + pos));
-                part[q] = x / scale[D.soff + (long long)mt * 128 + rho];
-            }
-            v = make_float2(part[0], part[1]);
-        }
-        out[e] = v;
+        out[e] = row >= 64 ? reinterpret_cast<const float2*>(tile + (size_t)TILE_UNIT * kw)[(size_t)(row - 64) * kw + kj]
+                           : reinterpret_cast<const float2*>(tile)[(size_t)kj * 64 + row];
     }
 }
 
@@ -477,18 +384,14 @@ constexpr int DT = 256;                 // compute threads (8 warps)
 constexpr int PT = 32;                  // the thread that issues the ring's copies (warp 1, lane 0)
 constexpr int DSTAGES = 2;              // operator tiles in flight
 constexpr int TILE_BYTES = 128 * 528;  // one ring stage: 128 K columns x (512 + 2 extra rows x 8) bytes
-constexpr int PSTR = 132;               // partial-sum row stride in floats (re/im interleaved, TC forms;
-                                        // 132 = 4 mod 32 banks: 16-byte stores of 8 rows hit distinct banks)
-constexpr int BBUF_BYTES = 128 * PSTR * 4;   // B operand, then the partial sums
+constexpr int BBUF_BYTES = 128 * 64 * 8;     // the input slice [128][64], then the partial sums [64][64]
 constexpr int PF_AHEAD = 4;             // tiles prefetched into L2 ahead of the ring
 constexpr long long DEFAULT_WAIT = 4000000000ll;   // about 2 s at 2 GHz
-// shared memory before the per-slab tables: ring, B / partials, column scales,
-// gather plan, column maxima, extra-row partials, update operands, barriers,
-// flags and the tile walk
-constexpr int DENSE_SMEM_FIXED = DSTAGES * TILE_BYTES + BBUF_BYTES + 128 * 4 + 128 * 4 + 128 * 4 + 2 * 64 * 8 +
-                                 3 * 256 * 8 + (DSTAGES + 3) * 8 + 16 + 2 * 48;
-
-enum { FORM_FP32 = 0, FORM_SPLIT = 1, FORM_HI = 2 };
+// shared memory before the per-slab tables: ring, input slice / partials, gather
+// plan, extra-row partials, update operands, barriers, flags and the tile walk
+constexpr int DENSE_SMEM_FIXED = DSTAGES * TILE_BYTES + BBUF_BYTES + 128 * 4 + 2 * 64 * 8 + 3 * 256 * 8 +
+                                 (DSTAGES + 2) * 8 + 16 + 2 * 48;
+constexpr int DENSE_MAX_B = 172;        // blocks per axis the dense forms take (n = 165 with b = 6, d = 1)
 
 // Work space of one apply launch (R8 right-hand sides, right-hand side fastest):
 //   V   [N lines][Wmax z rows][N x][R8]   forward values of the current slab
@@ -502,7 +405,6 @@ struct DenseArgs {
     const AxisWin* win;
     const DProb* dp;
     const unsigned char* G;
-    const float* scale;
     const float2* c_dn;
     const float2* c_up;
     const float2* rin;
@@ -516,10 +418,7 @@ struct DenseArgs {
     int nrhs, R8, nclus, nsteps, DZ;
     long long wait_cycles;
     int unmet;
-    int unit;
 };
-
-
 
 __device__ __forceinline__ int vbase(const DenseArgs& A, int line, int lz, int x) {
     return ((line * A.g.Wmax + lz) * A.g.N + x) * A.R8;
@@ -602,7 +501,7 @@ struct TileIter {
     }
     __device__ const unsigned char* ptr(const DenseArgs& A, int rank, uint32_t* bytes) const {
         const int kw = min(128, KR - 128 * c);
-        const int ux = A.unit + 8 * xr;
+        const int ux = TILE_UNIT + 8 * xr;
         *bytes = (uint32_t)(kw * ux);
         return A.G + off + ((long long)(mt * HELM_DENSE_CS + rank) * KR + 128 * c) * ux;
     }
@@ -647,32 +546,27 @@ __device__ __forceinline__ float2 gather_val(const DenseArgs& A, const int* s_sr
 
 // TWO: the sweep schedule (0 one front, 1 two fronts) as a compile-time constant:
 // the one-front kernel carries none of the two-front step mapping.
-template <int FORM, int TWO>
+template <int TWO>
 __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseArgs A) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int B = A.g.B;
     unsigned char* ring = smem;
     unsigned char* Bbuf = smem + DSTAGES * TILE_BYTES;
-    float* colsc = reinterpret_cast<float*>(Bbuf + BBUF_BYTES);      // [128] inverse column scales
-    int* s_src = reinterpret_cast<int*>(colsc + 128);                // [128] gather plan
-    unsigned* s_cmax = reinterpret_cast<unsigned*>(s_src + 128);     // [128] column maxima (float bits)
-    float2* s_xp = reinterpret_cast<float2*>(s_cmax + 128);          // [2][64] extra rows' partial sums
+    int* s_src = reinterpret_cast<int*>(Bbuf + BBUF_BYTES);          // [128] gather plan
+    float2* s_xp = reinterpret_cast<float2*>(s_src + 128);           // [2][64] extra rows' partial sums
     float2* s_pre = s_xp + 2 * 64;                                   // [3][DT] update operands (cp.async)
     uint64_t* full = reinterpret_cast<uint64_t*>(s_pre + 3 * DT);
-    uint64_t* mma_bar = full + DSTAGES;
-    uint64_t* ready = mma_bar + 1;         // every rank's partial sums are in place (8 arrivals)
+    uint64_t* ready = full + DSTAGES;      // every rank's partial sums are in place (8 arrivals)
     uint64_t* done = ready + 1;            // every rank has read the partial sums (8 arrivals)
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
-    volatile int* s_stop = reinterpret_cast<volatile int*>(tslot + 1);
+    volatile int* s_stop = reinterpret_cast<volatile int*>(done + 1);
     volatile int* s_issued = s_stop + 1;   // tiles issued into the ring
     volatile int* s_pend = s_issued + 1;   // released stages whose refill waits for the next step
-    TileIter<TWO>* s_itr = reinterpret_cast<TileIter<TWO>*>(tslot + 4);   // [2] fill, prefetch (8-byte aligned)
+    TileIter<TWO>* s_itr = reinterpret_cast<TileIter<TWO>*>(const_cast<int*>(s_stop) + 4);   // [2] fill, prefetch (8-byte aligned)
     static_assert(sizeof(TileIter<TWO>) <= 48, "the tile walk's shared slot");
     DProb* s_dp = reinterpret_cast<DProb*>(smem + DENSE_SMEM_FIXED);  // [B+1] operators of the current slab
     AxisWin* s_win = reinterpret_cast<AxisWin*>(s_dp + (B + 2));      // [B] windows
 
-    constexpr bool TC = FORM != FORM_FP32;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x;
     uint32_t rank;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     const int cid = blockIdx.x / HELM_DENSE_CS;
@@ -683,7 +577,6 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
         for (int q = 0; q < DSTAGES; ++q) {
             ptx::mbar_init(&full[q], 1);
         }
-        ptx::mbar_init(mma_bar, 1);
         ptx::mbar_init(ready, HELM_DENSE_CS);
         ptx::mbar_init(done, HELM_DENSE_CS);
         *s_stop = 0;
@@ -692,19 +585,10 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
         ptx::fence_mbar_init();
     }
     for (int q = tid; q < B; q += DT) s_win[q] = A.win[q];
-    if (TC && warp == 0) {
-        ptx::tmem_alloc(tslot, 256);
-        ptx::tmem_relinquish();
-    }
-    ptx::tc_fence_before();
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    ptx::tc_fence_after();
-    const uint32_t tmem = TC ? *tslot : 0u;
 
     int consumed = 0;                      // ring tiles seen landed by thread 0
     int tab_jo = -1;                       // the slab visit whose operator table is in s_dp
-    uint32_t mph = 0;                      // mma_bar phase
-    bool mma_pending = false;
     // Thread PT keeps the ring full: tile t goes into stage t mod DSTAGES once the
     // stage's previous tile is released, and one more tile is prefetched into L2
     // PF_AHEAD tiles ahead.  A release whose next tile belongs to a later step is
@@ -743,9 +627,6 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
         // ---------------- compute warps ----------------
         int stg = 0;
         uint32_t sph = 0, rph = 0, dph = 0;
-        const uint32_t idesc_all = ptx::umma_idesc_f16(128, 4 * R8);
-        const uint32_t idesc_hi = ptx::umma_idesc_f16(128, 2 * R8);
-        const int TPR = DT / R8;           // TC gather: threads per right-hand side (R8 a power of 2)
         const size_t NN = (size_t)N * N;
         for (int s = 0; s < A.nsteps; ++s) {
             const StepInfo si = step_info(s, B, A.g.cen, TWO, cid, A.nclus);
@@ -825,28 +706,10 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
             const int mi = tid / (R8 / 2), mrhs = 2 * (tid - mi * (R8 / 2));
             const int xown = HELM_DENSE_CS - 1 - (int)rank;
             int4 plm = make_int4(-1, -1, -1, -1), plx = make_int4(-1, -1, -1, -1);
-            // Row scales (powers of two).  The partial sums of complex row i are kept in
-            // units of s_min(i), the smaller scale of its real-part and imaginary-part
-            // tile rows: a tile row rho read back from TMEM is multiplied by s_min /
-            // s_rho (exact), the summed row by 1 / s_min.  Deferring 1 / s_min to after
-            // the sum keeps the partials in the normal FP32 range for tiny right-hand
-            // sides.
-            float sc_self = 1.f, sc_part = 1.f, sc_y0 = 1.f, sc_y1 = 1.f;
-            // This thread's plans and row scales for output tile mt (static data).
+            // This thread's plans for output tile mt (static data).
             auto tile_plans = [&](int mt) {
                 if (tid < 4 * R8) plm = row_plan(rows * mt + 8 * (int)rank + mi, &z2m);
                 if (xown < xr && tid < R8) plx = row_plan(rows * mt + 64 + xown, &z2x);
-                if (TC) {
-                    const float* sc = A.scale + D.soff + (long long)mt * 128;
-                    const int rt = 32 * (warp & 3) + lane;
-                    sc_self = __ldg(sc + rt);
-                    sc_part = __ldg(sc + (rt ^ 16));
-                    if (tid < 4 * R8) {
-                        const int rr = 8 * (int)rank + mi;
-                        sc_y0 = __ldg(sc + tile_row(rr, 0));
-                        sc_y1 = __ldg(sc + tile_row(rr, 1));
-                    }
-                }
             };
             // The update operands of those rows, fetched asynchronously: forward values
             // of the block (a backward solve; written by its forward solve, two or more
@@ -871,18 +734,16 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
                 ptx::cp_async_commit();
             };
             // ---- prologue: the first tile's plans and the chunk-0 gather plan are made
-            //      while thread 0 waits for step s-1 (single-chunk TC steps and all SIMT
-            //      steps; multi-chunk TC steps plan inline).  The update operands are
-            //      fetched here too unless step s-1 is the boundary phase that writes
-            //      them (then after the wait). ----
-            const bool pro = !si.phase && mcid < n_mt && !(TC && nkc > 1);
+            //      while thread 0 waits for step s-1.  The update operands are fetched here
+            //      too unless step s-1 is the boundary phase that writes them (then after the
+            //      wait). ----
+            const bool pro = !si.phase && mcid < n_mt;
             // (two fronts: the upper front's last forward solve reads the centre line the
             // lower front wrote one step before)
             const bool pre_early = si.k >= 2 && !(TWO && o.id == 0 && o.ry == ROLE_U && o.Mp == cen + 1 && cen_one);
             if (pro) {
                 tile_plans(mcid);
                 if (pre_early) fetch_pre();
-                if (TC && tid < 2 * R8) s_cmax[tid] = 0u;
                 gather_plan(A, D, o, wz, yb0, yb1, (int)rank * KR, min(128, KR), s_src, tid);
             }
             if (tid == PT && *s_pend > 0 && !*s_stop) {
@@ -1028,7 +889,7 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
             for (int mt = mcid; mt < n_mt; mt += mncl) {
                 const bool first = (mt == mcid);
                 if (!first || !pro) {
-                    // a later tile of this step (or a multi-chunk step): plans inline
+                    // a later tile of this step: plans inline
                     named_sync_compute();
                     tile_plans(mt);
                     fetch_pre();
@@ -1044,169 +905,8 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
                 for (int c = 0; c < nkc; ++c) {
                     const int kw = min(128, KR - 128 * c);
                     const int k0 = (int)rank * KR + 128 * c;
-                    const int nkg = kw / 8;
                     const bool planned = first && pro && c == 0;   // the prologue made this chunk's plan
-                    if (TC) {
-                        // ---- q slice -> FP16 hi + lo B tile, one power-of-two scale per column ----
-                        // thread (rhs = tid % R8, sub = tid / R8) takes K groups sub, sub + TPR, ...
-                        const int rhs = tid % R8, sub = tid / R8;
-                        if (!planned) {
-                        if (c == 0) {
-                            if (tid < 2 * R8) s_cmax[tid] = 0u;
-                            if (nkc > 1) {
-                                // several chunks share the accumulator: the column scale spans them all
-                                float mre = 0.f, mim = 0.f;
-                                for (int cc = 0; cc < nkc; ++cc) {
-                                    named_sync_compute();
-                                    gather_plan(A, D, o, wz, yb0, yb1, (int)rank * KR + 128 * cc,
-                                                min(128, KR - 128 * cc), s_src, tid);
-                                    named_sync_compute();
-                                    for (int kg = sub; kg < 16; kg += TPR)
-#pragma unroll
-                                        for (int e = 0; e < 8; ++e) {
-                                            const float2 v = gather_val(A, s_src, 8 * kg + e, rhs);
-                                            mre = fmaxf(mre, fabsf(v.x));
-                                            mim = fmaxf(mim, fabsf(v.y));
-                                        }
-                                }
-                                atomicMax(&s_cmax[rhs], __float_as_uint(mre));
-                                atomicMax(&s_cmax[R8 + rhs], __float_as_uint(mim));
-                            }
-                        }
-                        named_sync_compute();
-                        gather_plan(A, D, o, wz, yb0, yb1, k0, kw, s_src, tid);
-                        named_sync_compute();
-                        }
-                        float2 qv[4][8];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            // only the K groups of this chunk issue loads (kw = 64: two of the
-                            // four), so the ones that count are in flight together
-                            const int kg = min(sub + u * TPR, 15);
-                            if (sub + u * TPR < nkg) {
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) qv[u][e] = gather_val(A, s_src, 8 * kg + e, rhs);
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) qv[u][e] = make_float2(0.f, 0.f);
-                            }
-                        }
-                        if (nkc == 1) {
-                            float mre = 0.f, mim = 0.f;
-#pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                if (sub + u * TPR < nkg)
-#pragma unroll
-                                    for (int e = 0; e < 8; ++e) {
-                                        mre = fmaxf(mre, fabsf(qv[u][e].x));
-                                        mim = fmaxf(mim, fabsf(qv[u][e].y));
-                                    }
-                            atomicMax(&s_cmax[rhs], __float_as_uint(mre));
-                            atomicMax(&s_cmax[R8 + rhs], __float_as_uint(mim));
-                        }
-                        named_sync_compute();
-                        // each thread forms its own columns' scales from the maxima; colsc (the
-                        // inverses, read at the TMEM read-back) is written for later
-                        // (the maxima are non-negative floats: their bits order like the values; for
-                        // m > 0, frexp's exponent is the biased exponent field - 126, also for
-                        // subnormal m, where the clamp of scale_exp decides; 2^e is built from
-                        // its exponent field, exact for |e| <= 120)
-                        auto col_exp = [](unsigned bits) {
-                            return bits == 0u ? 0 : scale_exp((int)((bits >> 23) & 0xFFu) - 126);
-                        };
-                        const float sre = __int_as_float((col_exp(s_cmax[rhs]) + 127) << 23);
-                        const float sim = __int_as_float((col_exp(s_cmax[R8 + rhs]) + 127) << 23);
-                        if (c == 0 && tid < 2 * R8) colsc[tid] = __int_as_float((127 - col_exp(s_cmax[tid])) << 23);
-                        const int sbo = nkg * 128;
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int kg = sub + u * TPR;
-                            if (kg < nkg) {
-                                __align__(16) __half hr[8], lr[8], hm[8], lm[8];
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) {
-                                    const float xr = qv[u][e].x * sre, xi = qv[u][e].y * sim;
-                                    hr[e] = __float2half_rn(xr);
-                                    lr[e] = __float2half_rn(xr - __half2float(hr[e]));
-                                    hm[e] = __float2half_rn(xi);
-                                    lm[e] = __float2half_rn(xi - __half2float(hm[e]));
-                                }
-                                const size_t base = (size_t)kg * 128 + (rhs & 7) * 16;
-                                *reinterpret_cast<uint4*>(Bbuf + (size_t)(rhs >> 3) * sbo + base) =
-                                    *reinterpret_cast<const uint4*>(hr);
-                                *reinterpret_cast<uint4*>(Bbuf + (size_t)((R8 + rhs) >> 3) * sbo + base) =
-                                    *reinterpret_cast<const uint4*>(hm);
-                                *reinterpret_cast<uint4*>(Bbuf + (size_t)((2 * R8 + rhs) >> 3) * sbo + base) =
-                                    *reinterpret_cast<const uint4*>(lr);
-                                *reinterpret_cast<uint4*>(Bbuf + (size_t)((3 * R8 + rhs) >> 3) * sbo + base) =
-                                    *reinterpret_cast<const uint4*>(lm);
-                            }
-                        }
-                        ptx::fence_proxy_async_smem();
-                        // the tile must have landed: the MMA reads it, the extra rows are read below
-                        if (!wait_bar(&full[stg], sph, limit, false, nullptr)) {
-                            atomicOr(A.err, 2);
-                            *s_stop = 1;
-                        }
-                        named_sync_compute();
-                        const bool go = !*s_stop;          // the same value in every thread after the sync
-                        if (tid == 0 && go) {
-                            ++consumed;
-                            ptx::tc_fence_after();
-                            const uint32_t a_hi = ptx::smem_u32(ring + (size_t)stg * TILE_BYTES);
-                            const uint32_t a_lo = a_hi + (uint32_t)(128 * kw * 2);
-                            const uint32_t b0 = ptx::smem_u32(Bbuf);
-                            const uint32_t sb = (uint32_t)sbo;
-                            for (int ks = 0; ks < kw / 16; ++ks)
-                                ptx::umma_f16(tmem, ptx::umma_desc(a_hi + 256u * ks, 128u, sb),
-                                              ptx::umma_desc(b0 + 256u * ks, 128u, sb), idesc_all,
-                                              (c > 0 || ks > 0) ? 1u : 0u);
-                            if (FORM == FORM_SPLIT)
-                                for (int ks = 0; ks < kw / 16; ++ks)
-                                    ptx::umma_f16(tmem, ptx::umma_desc(a_lo + 256u * ks, 128u, sb),
-                                                  ptx::umma_desc(b0 + 256u * ks, 128u, sb), idesc_hi, 1u);
-                            ptx::umma_commit(mma_bar);
-                        }
-                        if (go && xr > 0) {
-                            // the FP32 extra rows on the SIMT lanes while the tensor core runs
-                            const float2* X = reinterpret_cast<const float2*>(ring + (size_t)stg * TILE_BYTES +
-                                                                              (size_t)A.unit * kw);
-                            for (int ex = 0; ex < xr; ++ex) {
-                                float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
-#pragma unroll
-                                for (int u = 0; u < 4; ++u) {
-                                    const int kg = sub + u * TPR;
-                                    if (kg < nkg)
-#pragma unroll
-                                        for (int e = 0; e < 8; e += 2) {
-                                            cfma(a0, X[ex * kw + 8 * kg + e], qv[u][e]);
-                                            cfma(a1, X[ex * kw + 8 * kg + e + 1], qv[u][e + 1]);
-                                        }
-                                }
-                                atomicAdd(&s_xp[ex * 64 + rhs].x, a0.x + a1.x);
-                                atomicAdd(&s_xp[ex * 64 + rhs].y, a0.y + a1.y);
-                            }
-                        }
-                        if (++stg == DSTAGES) { stg = 0; sph ^= 1u; }
-                        if (!go) break;
-                        // B is rewritten by the next chunk and TMEM is read after the last
-                        if (wait_bar(mma_bar, mph, limit, false, nullptr)) {
-                            mph ^= 1u;
-                        } else {
-                            atomicOr(A.err, 2);
-                            *s_stop = 1;
-                            mma_pending = true;            // teardown waits for it again
-                        }
-                        ptx::tc_fence_after();
-                        named_sync_compute();
-                        // the MMA and the extra rows are done with the stage: refill it now if
-                        // this step still needs the tile that goes there, else at the next step
-                        if (tid == PT && !*s_stop) {
-                            if (tiles_left(mt, c) >= DSTAGES) refill();
-                            else *s_pend = *s_pend + 1;
-                        }
-                        if (*s_stop) break;
-                    } else {
+                    {
                         // ---- SIMT: q slice as complex FP32 [kw][64], then the tile product ----
                         if (!planned) {
                             named_sync_compute();
@@ -1252,7 +952,7 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
                         }
                         if (xr > 0) {
                             const float2* X = reinterpret_cast<const float2*>(ring + (size_t)stg * TILE_BYTES +
-                                                                              (size_t)A.unit * kw);
+                                                                              (size_t)TILE_UNIT * kw);
                             const int rr = tid & 63, kq2 = tid >> 6;
                             for (int ex = 0; ex < xr; ++ex) {
                                 float2 acc2 = make_float2(0.f, 0.f);
@@ -1273,95 +973,7 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
                 // the update operands fetched asynchronously with the plans
                 ptx::cp_async_wait_all();
                 // ---- this rank's partial sums into Bbuf ----
-                if (TC) {
-                    // Warp (qd, hp) reads TMEM lanes 32 qd.. (tile rows) for right-hand sides
-                    // hp R8/2 .. (all of them in warps 0-3 when R8 = 8).  Per right-hand side
-                    // j: the row times q's real part, hi + lo, in columns j and 2 R8 + j,
-                    // times q's imaginary part in R8 + j and 3 R8 + j.  Lane l holds part
-                    // (l / 16) of complex row i = 16 qd + l mod 16: the real part contributes
-                    // (x, y) to Y_i = G_i q, the imaginary part (-y, x); lanes l and l ^ 16
-                    // add their contributions with one shuffle, each keeping half of the
-                    // right-hand sides, and store (re, im) pairs.
-                    float* Pp = reinterpret_cast<float*>(Bbuf);
-                    const int qd = warp & 3, hp = warp >> 2;
-                    const bool imp = (lane & 16) != 0;
-                    const float tfac = fminf(sc_self, sc_part) / sc_self;
-                    const uint32_t tb = tmem + ((uint32_t)(32 * qd) << 16);
-                    const int nh = R8 >= 16 ? R8 / 2 : (hp == 0 ? R8 : 0);
-                    const int j0 = R8 >= 16 ? hp * (R8 / 2) : 0;
-                    float* prow = Pp + (16 * qd + (lane & 15)) * PSTR;
-                    if (nh >= 16) {
-                        for (int jb = j0; jb < j0 + nh; jb += 16) {
-                            float hre[16], him[16], lre[16], lim[16];
-                            ptx::tmem_ld16(tb + (uint32_t)jb, hre);
-                            ptx::tmem_ld16(tb + (uint32_t)(R8 + jb), him);
-                            ptx::tmem_ld16(tb + (uint32_t)(2 * R8 + jb), lre);
-                            ptx::tmem_ld16(tb + (uint32_t)(3 * R8 + jb), lim);
-                            ptx::tmem_wait_ld();
-                            ptx::reg_tie16(hre);
-                            ptx::reg_tie16(him);
-                            ptx::reg_tie16(lre);
-                            ptx::reg_tie16(lim);
-                            float tx[16], ty[16];
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) {
-                                const float x = (hre[e] + lre[e]) * colsc[jb + e] * tfac;
-                                const float y = (him[e] + lim[e]) * colsc[R8 + jb + e] * tfac;
-                                tx[e] = imp ? -y : x;
-                                ty[e] = imp ? x : y;
-                            }
-                            // lane keeps right-hand sides jb + 8 imp .. + 7
-                            float ox[8], oy[8];
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) {
-                                const float sx = imp ? tx[e] : tx[8 + e], sy = imp ? ty[e] : ty[8 + e];
-                                const float rx_ = __shfl_xor_sync(0xffffffffu, sx, 16);
-                                const float ry_ = __shfl_xor_sync(0xffffffffu, sy, 16);
-                                ox[e] = (imp ? tx[8 + e] : tx[e]) + rx_;
-                                oy[e] = (imp ? ty[8 + e] : ty[e]) + ry_;
-                            }
-                            const int jk = jb + (imp ? 8 : 0);
-#pragma unroll
-                            for (int e = 0; e < 8; e += 2)
-                                *reinterpret_cast<float4*>(prow + 2 * (jk + e)) =
-                                    make_float4(ox[e], oy[e], ox[e + 1], oy[e + 1]);
-                        }
-                    } else if (nh == 8) {
-                        float hre[8], him[8], lre[8], lim[8];
-                        ptx::tmem_ld8(tb + (uint32_t)j0, hre);
-                        ptx::tmem_ld8(tb + (uint32_t)(R8 + j0), him);
-                        ptx::tmem_ld8(tb + (uint32_t)(2 * R8 + j0), lre);
-                        ptx::tmem_ld8(tb + (uint32_t)(3 * R8 + j0), lim);
-                        ptx::tmem_wait_ld();
-                        ptx::reg_tie8(hre);
-                        ptx::reg_tie8(him);
-                        ptx::reg_tie8(lre);
-                        ptx::reg_tie8(lim);
-                        float tx[8], ty[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float x = (hre[e] + lre[e]) * colsc[j0 + e] * tfac;
-                            const float y = (him[e] + lim[e]) * colsc[R8 + j0 + e] * tfac;
-                            tx[e] = imp ? -y : x;
-                            ty[e] = imp ? x : y;
-                        }
-                        float ox[4], oy[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float sx = imp ? tx[e] : tx[4 + e], sy = imp ? ty[e] : ty[4 + e];
-                            const float rx_ = __shfl_xor_sync(0xffffffffu, sx, 16);
-                            const float ry_ = __shfl_xor_sync(0xffffffffu, sy, 16);
-                            ox[e] = (imp ? tx[4 + e] : tx[e]) + rx_;
-                            oy[e] = (imp ? ty[4 + e] : ty[e]) + ry_;
-                        }
-                        const int jk = j0 + (imp ? 4 : 0);
-#pragma unroll
-                        for (int e = 0; e < 4; e += 2)
-                            *reinterpret_cast<float4*>(prow + 2 * (jk + e)) =
-                                make_float4(ox[e], oy[e], ox[e + 1], oy[e + 1]);
-                    }
-                    ptx::tc_fence_before();
-                } else {
+                {
                     float2* Pp = reinterpret_cast<float2*>(Bbuf);
                     const int rg = tid >> 4, cg = tid & 15;
 #pragma unroll
@@ -1384,8 +996,7 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
                 float4 rv[HELM_DENSE_CS];
                 if (main_ok) {
                     const int row = 8 * (int)rank + mi;
-                    const float* src = TC ? reinterpret_cast<const float*>(Bbuf) + row * PSTR + 2 * mrhs
-                                          : reinterpret_cast<const float*>(Bbuf) + 2 * (row * 64 + mrhs);
+                    const float* src = reinterpret_cast<const float*>(Bbuf) + 2 * (row * 64 + mrhs);
 #pragma unroll
                     for (int q = 0; q < HELM_DENSE_CS; ++q) rv[q] = ptx::ld_dsmem_f32x4(ptx::mapa(src, (uint32_t)q));
                 }
@@ -1405,11 +1016,6 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
                         y.z += rv[q].z;
                         y.w += rv[q].w;
                     }
-                    const float yinv = 1.f / fminf(sc_y0, sc_y1);
-                    y.x *= yinv;
-                    y.y *= yinv;
-                    y.z *= yinv;
-                    y.w *= yinv;
                     const float2 Y0 = make_float2(y.x, y.y), Y1 = make_float2(y.z, y.w);
                     const int4 pl = plm;
                     if (pl.x >= 0) {
@@ -1488,12 +1094,6 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
             wait_bar(&full[q], ph, limit, false, nullptr);
             if (++q == DSTAGES) { q = 0; ph ^= 1u; }
         }
-        if (TC && mma_pending) wait_bar(mma_bar, mph, limit, false, nullptr);
-    }
-    if (TC) {
-        ptx::tc_fence_before();
-        named_sync_compute();
-        if (warp == 0) ptx::tmem_dealloc(tmem, 256);
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -1502,17 +1102,8 @@ size_t dense_smem_bytes(int B) {
     return (size_t)DENSE_SMEM_FIXED + (size_t)(B + 2) * sizeof(DProb) + (size_t)B * sizeof(AxisWin);
 }
 
-template <int FORM>
-const void* dense_kernel(int sched) {
-    return sched == HELM_TWO_FRONT ? (const void*)k_dense<FORM, 1> : (const void*)k_dense<FORM, 0>;
-}
-
-const void* dense_kernel_for(int precision, int sched) {
-    switch (precision) {
-        case HELM_SPLIT_FP16: return dense_kernel<FORM_SPLIT>(sched);
-        case HELM_FP16: return dense_kernel<FORM_HI>(sched);
-        default: return dense_kernel<FORM_FP32>(sched);
-    }
+const void* dense_kernel_for(int sched) {
+    return sched == HELM_TWO_FRONT ? (const void*)k_dense<1> : (const void*)k_dense<0>;
 }
 
 }  // namespace
@@ -1521,12 +1112,11 @@ const void* dense_kernel_for(int precision, int sched) {
 
 // The operator table: sizes, index sets and storage offsets.
 static void build_dense_table(helm_ctx* h, const std::vector<AxisWin>& win, int nclus, std::vector<DProb>& out,
-                              size_t* gbytes, size_t* nscale) {
+                              size_t* gbytes) {
     const int B = h->g.B, N = h->g.N, b = h->g.b;
     const bool two = h->g.sched == HELM_TWO_FRONT;
-    const int unit = tile_unit(h->opts.precision);
     out.assign((size_t)dense_nops(B), DProb());
-    size_t off = 0, soff = 0;
+    size_t off = 0;
     for (int p = 0; p < dense_nops(B); ++p) {
         DProb D;
         memset(&D, 0, sizeof(D));
@@ -1579,13 +1169,10 @@ static void build_dense_table(helm_ctx* h, const std::vector<AxisWin>& win, int 
         D.KR = 16 * ceil_div(ceil_div(D.n_in, HELM_DENSE_CS), 16);
         D.nkc = ceil_div(D.KR, 128);
         D.off = (long long)off;
-        D.soff = (long long)soff;
-        off += (size_t)D.n_mt * HELM_DENSE_CS * D.KR * (unit + 8 * D.xr);
-        if (h->opts.precision != HELM_FP32) soff += (size_t)D.n_mt * 128;
+        off += (size_t)D.n_mt * HELM_DENSE_CS * D.KR * (TILE_UNIT + 8 * D.xr);
         out[p] = D;
     }
     *gbytes = off;
-    *nscale = soff;
 }
 
 // Factors and restricted operators of slabs Ma..Mb, for the line blocks
@@ -1616,6 +1203,8 @@ static int dense_build(helm_ctx* h, const Prob* prob, int Ma, int Mb, int Pa, in
     size_t fac_cap = 0, gt_cap = 0;
     GItem* d_items = nullptr;
     PItem* d_pitems = nullptr;
+    void* d_tpack = nullptr;
+    size_t tpack_cap = 0;
     long long* d_goff = nullptr;
     size_t items_cap = 0, pitems_cap = 0;
     int rc = HELM_OK;
@@ -1658,6 +1247,7 @@ static int dense_build(helm_ctx* h, const Prob* prob, int Ma, int Mb, int Pa, in
         // work items and temporary operator offsets of the chunk
         std::vector<GItem> items;
         std::vector<PItem> pitems;
+        std::vector<int> ops;
         long long go = 0;
         for (int M = M0; M < M1; ++M) {
             for (int q = 0; q <= B + 1; ++q) {
@@ -1668,7 +1258,10 @@ static int dense_build(helm_ctx* h, const Prob* prob, int Ma, int Mb, int Pa, in
                 goff[p] = go;
                 go += (long long)dp[p].n_out * dp[p].n_in;
                 for (int j0 = 0; j0 < dp[p].n_in; j0 += GW) items.push_back(GItem{p, j0});
-                for (int mt = 0; mt < dp[p].n_mt; ++mt) pitems.push_back(PItem{p, mt});
+                if (h->opts.precision == HELM_FP32)
+                    for (int mt = 0; mt < dp[p].n_mt; ++mt) pitems.push_back(PItem{p, mt});
+                else
+                    ops.push_back(p);
             }
         }
         if (items.size() > items_cap) {
@@ -1677,35 +1270,28 @@ static int dense_build(helm_ctx* h, const Prob* prob, int Ma, int Mb, int Pa, in
             DTRY(cudaMalloc(&d_items, items.size() * sizeof(GItem)));
             items_cap = items.size();
         }
-        if (pitems.size() > pitems_cap) {
+        if (!pitems.empty() && pitems.size() > pitems_cap) {
             if (d_pitems) cudaFree(d_pitems);
             d_pitems = nullptr;
             DTRY(cudaMalloc(&d_pitems, pitems.size() * sizeof(PItem)));
             pitems_cap = pitems.size();
         }
         DTRY(cudaMemcpyAsync(d_items, items.data(), items.size() * sizeof(GItem), cudaMemcpyHostToDevice, st));
-        DTRY(cudaMemcpyAsync(d_pitems, pitems.data(), pitems.size() * sizeof(PItem), cudaMemcpyHostToDevice, st));
+        if (!pitems.empty())
+            DTRY(cudaMemcpyAsync(d_pitems, pitems.data(), pitems.size() * sizeof(PItem), cudaMemcpyHostToDevice, st));
         DTRY(cudaMemcpyAsync(d_goff, goff.data(), sizeof(long long) * P, cudaMemcpyHostToDevice, st));
         const int nblk = (int)std::min<size_t>(items.size(), (size_t)gblocks);
         k_dense_G<<<nblk, GT, gsm, st>>>(h->g, h->t, h->dprob, d_items, (int)items.size(), fac, off0, Gt, d_goff,
                                          yscr, yslot);
         h->launches++;
         DTRY(cudaGetLastError());
-        switch (h->opts.precision) {
-            case HELM_SPLIT_FP16:
-                k_dense_pack<HELM_SPLIT_FP16><<<(int)pitems.size(), 256, 0, st>>>(h->dprob, d_pitems, Gt, d_goff,
-                                                                                h->dG, h->dscale);
-                break;
-            case HELM_FP16:
-                k_dense_pack<HELM_FP16><<<(int)pitems.size(), 256, 0, st>>>(h->dprob, d_pitems, Gt, d_goff, h->dG,
-                                                                          h->dscale);
-                break;
-            default:
-                k_dense_pack<HELM_FP32><<<(int)pitems.size(), 256, 0, st>>>(h->dprob, d_pitems, Gt, d_goff, h->dG,
-                                                                          h->dscale);
+        if (h->opts.precision == HELM_FP32) {
+            k_dense_pack<<<(int)pitems.size(), 256, 0, st>>>(h->dprob, d_pitems, Gt, d_goff, h->dG);
+            h->launches++;
+            DTRY(cudaGetLastError());
+        } else {
+            DTRY(team_pack(h, ops.data(), (int)ops.size(), Gt, d_goff, &d_tpack, &tpack_cap, st));
         }
-        h->launches++;
-        DTRY(cudaGetLastError());
         // the host arrays above must outlive their copies
         DTRY(cudaStreamSynchronize(st));
         M0 = M1;
@@ -1715,6 +1301,7 @@ static int dense_build(helm_ctx* h, const Prob* prob, int Ma, int Mb, int Pa, in
     cudaFree(Gt);
     cudaFree(d_items);
     cudaFree(d_pitems);
+    cudaFree(d_tpack);
     cudaFree(d_goff);
 #undef DTRY
     return rc;
@@ -1728,9 +1315,10 @@ int dense_setup(helm_ctx* h, const void* win_host, const void* prob_host, cudaSt
     cudaError_t e;
     // ---- the apply launch: clusters of 8 CTAs, as many as can be resident (<= 16) ----
     h->dsmem = dense_smem_bytes(B);
-    if (h->dsmem > (size_t)227 * 1024) return HELM_ENOTSUP;
-    {
-        const void* kfn = dense_kernel_for(h->opts.precision, h->g.sched);
+    if (B > DENSE_MAX_B) return HELM_ENOTSUP;
+    const bool fp32 = h->opts.precision == HELM_FP32;
+    if (fp32) {
+        const void* kfn = dense_kernel_for(h->g.sched);
         e = ensure_dyn_smem(kfn, h->dsmem);
         if (e != cudaSuccess) { helm_set_cuda_error(e); return HELM_ECUDA; }
         cudaLaunchConfig_t cfg;
@@ -1751,15 +1339,26 @@ int dense_setup(helm_ctx* h, const void* win_host, const void* prob_host, cudaSt
         if (ncl < 1) return HELM_ENOTSUP;
         h->dclus = std::min(ncl, 16);
         if (h->opts.dense_clusters > 0) h->dclus = std::min(h->dclus, h->opts.dense_clusters);
+    } else {
+        const int rc = team_configure(h);
+        if (rc != HELM_OK) return rc;
     }
     std::vector<DProb> dp;
     size_t gbytes = 0, nscale = 0;
-    build_dense_table(h, win, h->dclus, dp, &gbytes, &nscale);
+    build_dense_table(h, win, h->dclus, dp, &gbytes);
+    if (!fp32) {
+        h->tprob_h = new TProb[P];
+        team_table(h, dp.data(), h->tprob_h, &gbytes, &nscale);
+    }
     h->dprob_h = new DProb[P];
     memcpy(h->dprob_h, dp.data(), sizeof(DProb) * P);
 #define DTRY(x) do { e = (x); if (e != cudaSuccess) { helm_set_cuda_error(e); return e == cudaErrorMemoryAllocation ? HELM_ENOMEM : HELM_ECUDA; } } while (0)
     DTRY(cudaMalloc(&h->dprob, sizeof(DProb) * P));
     DTRY(cudaMemcpyAsync(h->dprob, dp.data(), sizeof(DProb) * P, cudaMemcpyHostToDevice, st));
+    if (!fp32) {
+        DTRY(cudaMalloc(&h->tprob, sizeof(TProb) * P));
+        DTRY(cudaMemcpyAsync(h->tprob, h->tprob_h, sizeof(TProb) * P, cudaMemcpyHostToDevice, st));
+    }
     DTRY(cudaMalloc(&h->dG, gbytes));
     h->dG_bytes = gbytes;
     if (nscale) {
@@ -1768,7 +1367,7 @@ int dense_setup(helm_ctx* h, const void* win_host, const void* prob_host, cudaSt
     }
 #undef DTRY
     const int rc = dense_build(h, prob.data(), 0, B - 1, 0, B - 1, st);
-    if (rc != HELM_OK) return rc;
+    if (rc != HELM_OK || !fp32) return rc;
     int most = 0;
     for (int p = 0; p < P; ++p) most = std::max(most, dp[p].n_mt);
     // two fronts run two solves side by side: at least two clusters, up to twice the tiles
@@ -1791,16 +1390,23 @@ static int dense_dz(const helm_ctx* h) {
     return std::max(h->g.b, h->g.sched == HELM_TWO_FRONT ? 2 * h->g.d : h->g.d);   // two fronts: the centre <= 2d
 }
 
-size_t dense_work_elems(const helm_ctx* h, int nrhs) {
+// Work space of the FP32 form; also the bound that helm_apply_precond_noalloc puts on every dense form.
+size_t dense_noalloc_elems(const helm_ctx* h, int nrhs) {
     // V, Q, Gv and Zv for one launch group (<= 64 right-hand sides), then the step counter (16 bytes)
     const size_t r8 = (size_t)dense_r8(std::min(nrhs, 64));
     const size_t NN = (size_t)h->g.N * h->g.N;
     return 2 * NN * h->g.Wmax * r8 + 2 * NN * dense_dz(h) * r8 + 2;
 }
 
-cudaError_t launch_dense_apply(helm_ctx* h, const float2* r, float2* z, int nrhs, float2* work, cudaStream_t st) {
+size_t dense_work_elems(const helm_ctx* h, int nrhs, size_t limit) {
+    return h->opts.precision == HELM_FP32 ? dense_noalloc_elems(h, nrhs) : team_work_elems(h, nrhs, limit);
+}
+
+cudaError_t launch_dense_apply(helm_ctx* h, const float2* r, float2* z, int nrhs, float2* work, size_t elems,
+                               cudaStream_t st) {
+    if (h->opts.precision != HELM_FP32) return launch_team_apply(h, r, z, nrhs, work, elems, st);
     const size_t n3 = (size_t)h->g.N * h->g.N * h->g.N;
-    const void* kfn = dense_kernel_for(h->opts.precision, h->g.sched);
+    const void* kfn = dense_kernel_for(h->g.sched);
     const size_t r8max = (size_t)dense_r8(std::min(nrhs, 64));
     const size_t NN = (size_t)h->g.N * h->g.N;
     float2* V = work;
@@ -1817,7 +1423,6 @@ cudaError_t launch_dense_apply(helm_ctx* h, const float2* r, float2* z, int nrhs
         A.win = h->t.win;
         A.dp = h->dprob;
         A.G = h->dG;
-        A.scale = h->dscale;
         A.c_dn = h->t.c_dn;
         A.c_up = h->t.c_up;
         A.rin = r + (size_t)r0 * n3;
@@ -1835,7 +1440,6 @@ cudaError_t launch_dense_apply(helm_ctx* h, const float2* r, float2* z, int nrhs
         A.DZ = dense_dz(h);
         A.wait_cycles = h->opts.wait_cycles;
         A.unmet = h->opts.debug_unmet_wait;
-        A.unit = tile_unit(h->opts.precision);
         cudaError_t e = cudaMemsetAsync(ctr, 0, sizeof(unsigned), st);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg;
@@ -1865,10 +1469,13 @@ int dense_rebuild(helm_ctx* h, int Ma, int Mb, int Pa, int Pb, cudaStream_t st) 
 }
 
 void dense_free(helm_ctx* h) {
-    void* ptrs[] = {h->dprob, h->dG, h->dscale, h->dV};
+    void* ptrs[] = {h->dprob, h->tprob, h->dG, h->dscale, h->dV};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete[] h->dprob_h;
+    delete[] h->tprob_h;
+    h->tprob = nullptr;
+    h->tprob_h = nullptr;
     h->dprob = nullptr;
     h->dprob_h = nullptr;
     h->dG = nullptr;
@@ -1899,13 +1506,14 @@ extern "C" int helm_dense_operator(helm_handle h, int M, int Mp, int dir, int* n
     }
     if (!G) return HELM_OK;
     cudaStream_t st = (cudaStream_t)stream;
-    switch (h->opts.precision) {
-        case HELM_SPLIT_FP16: k_dense_unpack<HELM_SPLIT_FP16><<<512, 256, 0, st>>>(D, h->dG, h->dscale, (float2*)G); break;
-        case HELM_FP16: k_dense_unpack<HELM_FP16><<<512, 256, 0, st>>>(D, h->dG, h->dscale, (float2*)G); break;
-        default: k_dense_unpack<HELM_FP32><<<512, 256, 0, st>>>(D, h->dG, h->dscale, (float2*)G);
+    cudaError_t e;
+    if (h->opts.precision == HELM_FP32) {
+        k_dense_unpack<<<512, 256, 0, st>>>(D, h->dG, (float2*)G);
+        h->launches++;
+        e = cudaGetLastError();
+    } else {
+        e = team_unpack(h, p, (float2*)G, st);
     }
-    h->launches++;
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         helm_set_cuda_error(e);
         return HELM_ECUDA;

@@ -64,6 +64,18 @@ struct DProb {
     long long soff;     // float offset of its per-row scales (FP16 forms)
 };
 
+// A stored operator of the tensor-core forms (team_map.h): the same index sets,
+// rows in groups of 8 per out rect, input columns padded to a multiple of 16.
+struct TProb {
+    int n_out, n_in;
+    DRect out[2], in;
+    int ng0, ng1;       // row groups of the out rects
+    int KP;             // padded input columns
+    int pad_;
+    long long off;      // byte offset of the operator's chunks
+    long long soff;     // float offset of its per-row scales (16 per group)
+};
+
 #define HELM_DENSE_CS 8   // CTAs per cluster in the dense apply (the K split)
 
 struct Geom {
@@ -142,7 +154,12 @@ struct helm_ctx {
     size_t dscale_elems;
     float2* dV;              // apply work space: slab vector [line][z row][x][64 RHS], then the op counter
     size_t dV_elems;
-    int dclus;               // clusters of HELM_DENSE_CS CTAs in the apply launch
+    int dclus;               // FP32 form: clusters of HELM_DENSE_CS CTAs in the apply launch;
+                             // tensor-core forms: CTAs it may use
+    TProb* tprob;            // tensor-core forms: the operator table on the device
+    TProb* tprob_h;          // and on the host
+    void* win_h;             // host copy of the axis windows (AxisWin[B])
+    int team_min_groups;     // least row groups of 8 per rank of a team
     size_t dsmem;            // dynamic shared memory of the apply kernel
 };
 
@@ -178,9 +195,21 @@ cudaError_t launch_factor_range(helm_ctx* h, int p0, int np, float2* dst, long l
 int dense_setup(helm_ctx* h, const void* win_host, const void* prob_host, cudaStream_t st);
 int dense_rebuild(helm_ctx* h, int Ma, int Mb, int Pa, int Pb, cudaStream_t st);
 cudaError_t sweep_prepare(helm_ctx* h, int nrhs, cudaStream_t st);
-cudaError_t launch_dense_apply(helm_ctx* h, const float2* r, float2* z, int nrhs, float2* work, cudaStream_t st);
-size_t dense_work_elems(const helm_ctx* h, int nrhs);
+// work: at least dense_work_elems(h, nrhs, elems) of the `elems` float2 there are
+cudaError_t launch_dense_apply(helm_ctx* h, const float2* r, float2* z, int nrhs, float2* work, size_t elems,
+                               cudaStream_t st);
+size_t dense_work_elems(const helm_ctx* h, int nrhs, size_t limit);
+size_t dense_noalloc_elems(const helm_ctx* h, int nrhs);
 void dense_free(helm_ctx* h);
+// Tensor-core forms of the dense apply (team.cu).
+void team_table(const helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t* nscale);
+cudaError_t team_pack(helm_ctx* h, const int* ops, int nops, const float2* Gt, const long long* d_goff,
+                      void** d_items, size_t* cap, cudaStream_t st);
+cudaError_t team_unpack(helm_ctx* h, int p, float2* G, cudaStream_t st);
+int team_configure(helm_ctx* h);
+size_t team_work_elems(const helm_ctx* h, int nrhs, size_t limit);
+cudaError_t launch_team_apply(helm_ctx* h, const float2* r, float2* z, int nrhs, float2* work, size_t elems,
+                              cudaStream_t st);
 cudaError_t launch_stencil_c64(helm_ctx* h, const float2* x, float2* y, int nrhs, cudaStream_t st);
 cudaError_t launch_stencil_c128(helm_ctx* h, const double2* x, double2* y, int nrhs, cudaStream_t st);
 cudaError_t launch_residual_c128(helm_ctx* h, const float2* f, const double2* u, double2* r,

@@ -38,6 +38,16 @@ __device__ __forceinline__ bool mbar_try_cluster(uint64_t* bar, uint32_t parity)
                  : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
     return ok != 0;
 }
+// Up to n polls of a phase in a tight loop; the barrier by its shared address.
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, uint32_t n) {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p, q;\n .reg .u32 i;\n mov.u32 i, %3;\n"
+                 "POLL_LOOP_%=:\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                 " @p bra POLL_DONE_%=;\n sub.u32 i, i, 1;\n setp.ne.u32 q, i, 0;\n @q bra POLL_LOOP_%=;\n"
+                 "POLL_DONE_%=:\n selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(n) : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -112,6 +122,36 @@ __device__ __forceinline__ void red_release_gpu_add(unsigned* p, unsigned v) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Relaxed (uncached) 16-byte load, and 8-byte store, at GPU scope: words another
+// CTA writes while this one polls them.
+__device__ __forceinline__ uint4 ld_relaxed_gpu_v4(const void* p) {
+    uint4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed_gpu_u64(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// Loads that stay where they are written (volatile): prefetches into registers
+// ahead of a wait.
+__device__ __forceinline__ float4 ld_cg_f32x4_here(const void* p) {
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_nc_f32_here(const float* p) {
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+// Orders this thread's view of global memory written by the generic proxy before
+// its later bulk copies (async proxy) of it.
+__device__ __forceinline__ void fence_proxy_async_global() {
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+}
+
 // ---- tcgen05 ------------------------------------------------------------------
 // TMEM allocation: one full warp, converged.  The address lands in *dst.
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t ncols) {
@@ -145,12 +185,30 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint
 __host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N) {
     return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
+// The same with B stored N-major (bit 16): 8 x 8 core matrices of 8 K rows x 16
+// bytes (8 N values); the descriptor's LBO then steps 8 K rows and its SBO 8 N
+// columns.
+__host__ __device__ constexpr uint32_t umma_idesc_f16_bn(int M, int N) { return umma_idesc_f16(M, N) | (1u << 16); }
 // D[tmem] (+)= A[smem] * B[smem]^T, issued by one thread.
 __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
                  ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// The same two from a converged warp: one lane is elected to issue, and with
+// operands equal in every lane the compiler keeps them in uniform registers
+// (about 30 cycles per product instead of 70 to 250 from a divergent branch).
+__device__ __forceinline__ void umma_f16_warp(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accumulate) {
+    asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n elect.sync _|q, 0xffffffff;\n"
+                 " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
+                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void umma_commit_warp(uint64_t* bar) {
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
+                 " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}"
+                 ::"r"(smem_u32(bar)) : "memory");
 }
 // Arrive once on `bar` when every MMA this thread issued so far has completed.
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
@@ -172,6 +230,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
                    "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]),
                    "=f"(v[15])
                  : "r"(taddr) : "memory");
+}
+// 16 lanes x 8 consecutive 32-bit columns spread over the warp: thread t gets
+// lane t/4, columns 2 (t mod 4) and + 1 in v[0], v[1], and lane t/4 + 8 in v[2],
+// v[3] (valid after tmem_wait_ld + reg_tie4).
+__device__ __forceinline__ void tmem_ld16x8(uint32_t taddr, float (&v)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void reg_tie4(float (&v)[4]) {
+    asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]));
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Placed after tmem_wait_ld (volatile statements keep their order): every use

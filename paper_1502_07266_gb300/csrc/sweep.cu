@@ -784,7 +784,7 @@ cudaError_t launch_sweep_batch(helm_ctx* const* hs, const float2* const* r, floa
 // captured into a CUDA graph.
 cudaError_t sweep_prepare(helm_ctx* h, int nrhs, cudaStream_t st) {
     if (h->dense) {
-        const size_t need = dense_work_elems(h, nrhs);
+        const size_t need = dense_work_elems(h, nrhs, (size_t)-1);
         if (need > h->dV_elems) {
             if (h->dV) cudaFree(h->dV);
             h->dV = nullptr;
@@ -808,7 +808,7 @@ cudaError_t launch_sweep(helm_ctx* h, const float2* r, float2* z, int nrhs, int 
                          cudaStream_t st) {
     if (h->dense) {
         if (slab_only) return cudaErrorNotSupported;
-        const size_t need = dense_work_elems(h, nrhs);
+        const size_t need = dense_work_elems(h, nrhs, (size_t)-1);
         if (need > h->dV_elems) {
             if (h->dV) cudaFree(h->dV);
             h->dV = nullptr;
@@ -817,7 +817,7 @@ cudaError_t launch_sweep(helm_ctx* h, const float2* r, float2* z, int nrhs, int 
             if (e != cudaSuccess) return e;
             h->dV_elems = need;
         }
-        return launch_dense_apply(h, r, z, nrhs, h->dV, st);
+        return launch_dense_apply(h, r, z, nrhs, h->dV, h->dV_elems, st);
     }
     cudaError_t e = ensure_slab(h, nrhs, st);
     if (e != cudaSuccess) return e;
@@ -845,15 +845,16 @@ extern "C" int helm_apply_precond_noalloc(helm_handle h, const void* r, void* z,
         return HELM_ECUDA;
     }
     if (dev != h->device) return HELM_EINVAL;             // the handle's factors live on another GPU
-    const size_t need = h->dense ? dense_work_elems(h, nrhs) : slab_need(h, nrhs);
-    if (need > HELM_NOALLOC_SCRATCH_BYTES / sizeof(float2)) return HELM_EINVAL;
+    const size_t room = HELM_NOALLOC_SCRATCH_BYTES / sizeof(float2);
+    const size_t need = h->dense ? dense_noalloc_elems(h, nrhs) : slab_need(h, nrhs);
+    if (need > room || (h->dense && dense_work_elems(h, nrhs, room) > room)) return HELM_EINVAL;
     void* scratch = nullptr;
     e = cudaGetSymbolAddress(&scratch, g_noalloc_scratch);
     if (e != cudaSuccess) {
         helm_set_cuda_error(e);
         return HELM_ECUDA;
     }
-    e = h->dense ? launch_dense_apply(h, (const float2*)r, (float2*)z, nrhs, static_cast<float2*>(scratch),
+    e = h->dense ? launch_dense_apply(h, (const float2*)r, (float2*)z, nrhs, static_cast<float2*>(scratch), room,
                                       (cudaStream_t)stream)
                  : launch_sweep_on(h, (const float2*)r, (float2*)z, nrhs, 0, 0, static_cast<float2*>(scratch),
                                    (cudaStream_t)stream);
