@@ -272,18 +272,25 @@ __device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t ph, long long
     }
 }
 
+// K = 16 steps of a part of a gather of n16 steps: whole operator chunks, so that a
+// chunk never waits for two parts.
+__device__ __forceinline__ int gather_part(int n16) {
+    constexpr int U = TKC / 16;
+    return (n16 + NBC * U - 1) / (NBC * U) * U;
+}
+
 // Y = G q of one row pair of right-hand sides from a tile's accumulators: in
 // each, the row's real parts (lane t/4) and imaginary parts (lane t/4 + 8) times
-// q's re hi, im hi, and the sums of the products with one lo part.  The
-// accumulators cover successive runs of input chunks and are added here in
-// rounded FP32 (the tensor core's own additions do not round to nearest: one
-// long chain costs accuracy).  er, ei: exponents of the row's scales; c0, c1: of
-// the columns'.
+// q's re hi, im hi, re lo, im lo; with split operators the products of their lo
+// parts with q's hi parts 16 lanes further on.  The accumulators cover successive
+// runs of input chunks and are added here in rounded FP32 (the tensor core's own
+// additions do not round to nearest: one long chain costs accuracy).  er, ei:
+// exponents of the row's scales; c0, c1: of the columns'.
 template <int RG>
-__device__ __forceinline__ float4 read_rows(uint32_t ta, int nacc, int er, int ei, int c0, int c1) {
+__device__ __forceinline__ float4 read_rows(uint32_t ta, int nacc, bool split, int er, int ei, int c0, int c1) {
     float R[4] = {0.f, 0.f, 0.f, 0.f}, I[4] = {0.f, 0.f, 0.f, 0.f};
     __syncwarp();                                    // the TMEM loads are warp-collective
-    float rh[NACC][4], mh[NACC][4], rl[NACC][4], ml[NACC][4];
+    float rh[NACC][4], mh[NACC][4], rl[NACC][4], ml[NACC][4], lr[NACC][4], lm[NACC][4];
 #pragma unroll
     for (int a = 0; a < NACC; ++a)
         if (a < nacc) {
@@ -291,6 +298,10 @@ __device__ __forceinline__ float4 read_rows(uint32_t ta, int nacc, int er, int e
             ptx::tmem_ld16x8(ta + a * 4 * RG + RG, mh[a]);
             ptx::tmem_ld16x8(ta + a * 4 * RG + 2 * RG, rl[a]);
             ptx::tmem_ld16x8(ta + a * 4 * RG + 3 * RG, ml[a]);
+            if (split) {
+                ptx::tmem_ld16x8(ta + (16u << 16) + a * 4 * RG, lr[a]);
+                ptx::tmem_ld16x8(ta + (16u << 16) + a * 4 * RG + RG, lm[a]);
+            }
         }
     ptx::tmem_wait_ld();
 #pragma unroll
@@ -300,6 +311,15 @@ __device__ __forceinline__ float4 read_rows(uint32_t ta, int nacc, int er, int e
             ptx::reg_tie4(mh[a]);
             ptx::reg_tie4(rl[a]);
             ptx::reg_tie4(ml[a]);
+            if (split) {
+                ptx::reg_tie4(lr[a]);
+                ptx::reg_tie4(lm[a]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    rl[a][q] += lr[a][q];
+                    ml[a][q] += lm[a][q];
+                }
+            }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 R[q] += rh[a][q] + rl[a][q];
@@ -318,6 +338,34 @@ __device__ __forceinline__ float4 read_rows(uint32_t ta, int nacc, int er, int e
 // 2^d (d <= 0) as FP16 bits; 0 below the subnormal range.
 __device__ __forceinline__ unsigned half_pow2(int d) {
     return d >= -14 ? (unsigned)(15 + d) << 10 : (d >= -24 ? 1u << (24 + d) : 0u);
+}
+
+// The products of one operator chunk (kc <= TKC input entries): one per 16 entries
+// and 4 row groups, all of one shape (only then do products into the same
+// accumulator keep their order).  With split operators a group's hi and lo rows
+// stand in the same product (128 rows: re hi, im hi, re lo, im lo of each group), which
+// takes 38 cycles where a 64-row product for hi and one for lo take 65; without, 64
+// rows.  One elected lane of the converged warp issues them; a full chunk is
+// straight-line code: a condition around each, even a uniform one, made a product
+// take 70 to 85 cycles to issue instead of 33.
+template <int RG, int NSUB>
+__device__ __forceinline__ void chunk_products(uint32_t d, uint64_t ad, uint32_t sub, uint64_t bd, uint32_t idesc, uint32_t add,
+                                               int kc) {
+    constexpr int BSTEP = 2 * 64 * RG / 16, ASTEP = 256 / 16, SUBC = NACC * 4 * RG;
+    if (kc == TKC) {
+#pragma unroll
+        for (int ks = 0; ks < TKC / 16; ++ks)
+#pragma unroll
+            for (int u = 0; u < NSUB; ++u)
+                ptx::umma_f16_warp(d + u * SUBC, ad + ks * ASTEP + u * sub, bd + ks * BSTEP, idesc, ks == 0 ? add : 1u);
+        return;
+    }
+#pragma unroll 1
+    for (int ks = 0; 16 * ks < kc; ++ks) {
+#pragma unroll
+        for (int u = 0; u < NSUB; ++u) ptx::umma_f16_warp(d + u * SUBC, ad + ks * ASTEP + u * sub, bd + ks * BSTEP, idesc, add);
+        add = 1u;
+    }
 }
 
 // What the roles of a CTA need to know of a solve's shape.  A visit has four kinds
@@ -417,8 +465,8 @@ struct Upd {
 // entry's words stay with one warp.
 template <int RG, int MT>
 __device__ __forceinline__ int warp_of(int gi, int pcb) {
-    if (RG == 16) return (MT == 64 ? gi & 3 : gi >> 1 & 3) + 4 * pcb;
-    return MT == 64 ? gi & 3 : (gi >> 1 & 3) + 4 * (gi & 1);
+    if (RG == 16) return (gi & 3) + 4 * pcb;
+    return MT == 64 ? gi & 3 : gi & 7;
 }
 // Where a lane's part of a row lies in its group of 8 entries, for right-hand sides
 // 8 pcb ..: part lane mod 4 (re hi, im hi, re lo, im lo) of row lane / 4.
@@ -464,13 +512,13 @@ __device__ __forceinline__ void publish(unsigned char* p, u64* hd, float4 v, int
 template <int RG, int MT>
 __device__ __noinline__ void clear_slot(unsigned char* xs, int kg0, int kg1) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll 1
-    for (int t = 0; t < (kg1 - kg0) * (RG / 8); ++t) {
-        const int gi = t / (RG / 8), pcb = t % (RG / 8);
-        if (warp_of<RG, MT>(gi, pcb) != warp) continue;
-        __stcg(reinterpret_cast<uint4*>(xs + (size_t)(kg0 + gi) * 64 * RG + part_offset<RG>(pcb, lane)),
+    constexpr int STEP = RG == 8 && MT == 128 ? 8 : 4;        // groups between a warp's own (warp_of)
+    const int pcb = RG == 16 ? warp >> 2 : 0;
+    const int gi = RG == 8 && MT == 64 && warp > 3 ? kg1 - kg0 : warp & (STEP - 1);
+#pragma unroll 4
+    for (int kg = kg0 + gi; kg < kg1; kg += STEP)
+        __stcg(reinterpret_cast<uint4*>(xs + (size_t)kg * 64 * RG + part_offset<RG>(pcb, lane)),
                make_uint4(STALE, STALE, STALE, STALE));
-    }
     __syncwarp();
 }
 
@@ -506,7 +554,7 @@ __device__ __noinline__ void boundary_phase(const TeamArgs& A, Sm* T, int jo) {
     const int wid = (T->team * T->C + T->rank) * CW + warp, nw = A.T * T->C * CW;
     const int nxb = (N + 7) >> 3, ntask = N * nxb * (RG / 4);
     // a warp task: 8 x of one line, 4 right-hand sides (whole 32-byte sectors on both sides)
-    constexpr int PP = 2;
+    constexpr int PP = 4;
 #pragma unroll 1
     for (int t0 = wid; t0 < ntask; t0 += PP * nw) {
         int gi_[PP], zx[PP], ls[PP], rr[PP];
@@ -591,13 +639,13 @@ __device__ __noinline__ void boundary_phase(const TeamArgs& A, Sm* T, int jo) {
 template <int RG, int MT>
 __device__ __noinline__ void general_rows(const TeamArgs& A, Sm* T, int M, int i, int tb, long long soff,
               uint32_t tmem, int ec0, int ec1) {
-    constexpr int GT = MT / 16, NRS = RG == 16 && MT == 128 ? 2 : 1, TCOLS = NACC * 4 * RG, TBATCH = 512 / TCOLS;
+    constexpr int GT = MT / 16, NRS = RG == 16 && MT == 128 ? 2 : 1, SUBC = NACC * 4 * RG, TCOLS = MT / 64 * SUBC, TBATCH = 512 / TCOLS;
     const int N = T->N, B = T->B, cen = T->cen, two = T->two, U = T->U, team = T->team, VL = T->VL, GL = T->GL;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q4 = warp & 3, hh = warp >> 2, ii = lane >> 2, c = lane & 3;
     const int cb = RG == 16 ? hh : 0, rhs0 = 8 * cb + 2 * c;
-    const int gi0 = MT == 64 ? q4 : (RG == 16 ? 2 * q4 : 2 * q4 + hh);
+    const int gi0 = RG == 8 && MT == 128 ? warp : q4;
     const bool idle = RG == 8 && MT == 64 && hh == 1;
-    const uint32_t tlane = tmem + ((uint32_t)(32 * q4 + (MT == 64 ? 0 : 16 * (gi0 & 1))) << 16) + 8 * cb;
+    const uint32_t tlane = tmem + ((uint32_t)(32 * q4) << 16) + 8 * cb + (gi0 >> 2) * SUBC;
     const int nsol = tm_solves(B, cen, team);
     const TeamSolve t = tm_solve(i, B, cen, team);
     const AxisWin wz = T->win[M], wy = T->win[t.Mp];
@@ -618,13 +666,13 @@ __device__ __noinline__ void general_rows(const TeamArgs& A, Sm* T, int M, int i
     for (int tl = tb; tl < min(S.nt, tb + TBATCH); ++tl)
 #pragma unroll 1
         for (int j = 0; j < NRS; ++j) {
-            const int pos = tl * GT + gi0 + j;
+            const int pos = tl * GT + gi0 + 4 * j;
             if (idle || pos >= S.c0 + S.c1) continue;      // the same in the whole warp
             const int rect = pos >= S.c0, gid = rect ? S.a1 + pos - S.c0 : S.a0 + pos;
             const int r = 8 * gid + ii;
             const int nl = rect ? g.out1.nl : g.out0.nl, nz = rect ? g.out1.nz : g.out0.nz;
             const float* sc = A.scale + soff + (long long)((rect ? S.ng0 : 0) + gid) * 16 + ii;
-            float4 X = read_rows<RG>(tlane + ((uint32_t)(16 * j) << 16) + (uint32_t)((tl - tb) * TCOLS), S.nacc,
+            float4 X = read_rows<RG>(tlane + (uint32_t)(j * SUBC + (tl - tb) * TCOLS), S.nacc, A.halves == 2,
                                      (__float_as_int(__ldg(sc)) >> 23) - 127,
                                      (__float_as_int(__ldg(sc + 8)) >> 23) - 127, ec0, ec1);
             if (r < (rect ? g.n1 : g.n0)) {
@@ -699,7 +747,7 @@ __device__ __forceinline__ bool validate(Sm& T, Upd& u, const unsigned char* xs,
     bool ok = true;
 #pragma unroll 1
     for (int k0 = 0; k0 < KP && ok; k0 += KB) {
-        const int n16 = (min(KP, k0 + KB) - k0) >> 4, part = (n16 + NBC - 1) / NBC;
+        const int n16 = (min(KP, k0 + KB) - k0) >> 4, part = gather_part(n16);
         const int vpart = part * (2 * KGB / 16);
         int left = n16 * (2 * KGB / 16), base = 0;
 #pragma unroll 1
@@ -710,16 +758,16 @@ __device__ __forceinline__ bool validate(Sm& T, Upd& u, const unsigned char* xs,
             uint4* b = reinterpret_cast<uint4*>(T.Bbuf) + base;
             int good = 1, wrote = 0;
 #pragma unroll 1
-            for (int v0 = tid; v0 < nvec; v0 += 4 * 32 * CW) {
-                unsigned m[4];
+            for (int v0 = tid; v0 < nvec; v0 += 8 * 32 * CW) {
+                unsigned m = 0u;
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
+                for (int r = 0; r < 8; ++r) {
                     const uint4 w = b[min(v0 + r * 32 * CW, nvec - 1)];
-                    m[r] = max(max(w.x, w.y), max(w.z, w.w));
+                    m = max(m, max(max(w.x, w.y), max(w.z, w.w)));
                 }
-                if (max(max(m[0], m[1]), max(m[2], m[3])) == STALE) {
+                if (m == STALE) {
 #pragma unroll 1
-                    for (int v = v0; v < min(nvec, v0 + 4 * 32 * CW); v += 32 * CW) {
+                    for (int v = v0; v < min(nvec, v0 + 8 * 32 * CW); v += 32 * CW) {
                         const uint4* src = reinterpret_cast<const uint4*>(xs + (size_t)k0 * (KGB / 8)) + base + v;
                         const long long t0 = clock64();
                         uint4 x = b[v];
@@ -848,20 +896,22 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
     const int ii = lane >> 2, c = lane & 3;               // row of a group, pair of right-hand sides
     const int cb = RG == 16 ? hh : 0;
     const int rhs0 = 8 * cb + 2 * c;                      // this thread's right-hand sides rhs0, rhs0 + 1
-    const int gi0 = MT == 64 ? q4 : (RG == 16 ? 2 * q4 : 2 * q4 + hh);   // its first row group of a tile
+    const int gi0 = RG == 8 && MT == 128 ? warp : q4;     // its first row group of a tile (the second: 4 on)
     const bool idle = RG == 8 && MT == 64 && hh == 1;     // no accumulator columns for this warp
-    const uint32_t tlane = T.tslot + ((uint32_t)(32 * q4 + (MT == 64 ? 0 : 16 * (gi0 & 1))) << 16) + 8 * cb;
+    constexpr int SUBC = NACC * 4 * RG;
+    const uint32_t tlane = T.tslot + ((uint32_t)(32 * q4) << 16) + 8 * cb + (gi0 >> 2) * SUBC;
+    const bool split = A.halves == 2;
     const int B = T.B, cen = T.cen, team = T.team, nsol = T.nsol;
     const AxisWin wz = T.win[pass_pos(jo, B, cen).M];
     const int Lz = wz.L, za = wz.ia, dz = wz.ib - wz.ia, E = T.N * Lz, KP = tm_kp(E);
     int cg0, cg1;                                         // this rank's groups of 8 columns
     tm_part(E, 1, 1, T.rank, T.C, &cg0, &cg1);
     cg0 += gi0;                                           // this warp's (first) group
-    const bool fv = !idle && cg0 < cg1, fv1 = NRS == 2 && cg0 + 1 < cg1;   // it exists (rows beyond E are zero)
+    const bool fv = !idle && cg0 < cg1, fv1 = NRS == 2 && cg0 + 4 < cg1;   // it exists (rows beyond E are zero)
     int fe[NRS], fz[NRS];                                 // column and own-layer offsets (-1: none) per row set
 #pragma unroll
     for (int j = 0; j < NRS; ++j) {
-        const int e = 8 * (cg0 + j) + ii, x = e / Lz, lz = e - x * Lz;
+        const int e = 8 * (cg0 + 4 * j) + ii, x = e / Lz, lz = e - x * Lz;
         fe[j] = (j ? fv1 : fv) && e < E ? e * RG + rhs0 : -1;
         fz[j] = fe[j] >= 0 && lz >= za && lz < za + dz ? (x * dz + lz - za) * RG + rhs0 : -1;
     }
@@ -897,8 +947,8 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
             pre[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             er[j] = ei[j] = 0;
             if (fe[j] >= 0) {
-                er[j] = __float_as_int(ptx::ld_nc_f32_here(sc + 16 * j));
-                ei[j] = __float_as_int(ptx::ld_nc_f32_here(sc + 16 * j + 8));
+                er[j] = __float_as_int(ptx::ld_nc_f32_here(sc + 64 * j));
+                ei[j] = __float_as_int(ptx::ld_nc_f32_here(sc + 64 * j + 8));
             }
             const int o = bwd ? fe[j] : fz[j];
             if (o >= 0) pre[j] = ptx::ld_cg_f32x4_here((bwd ? line : gl) + o);
@@ -916,7 +966,7 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
 #pragma unroll
         for (int j = 0; j < NRS; ++j)
             if (j ? fv1 : fv)
-                W[j] = read_rows<RG>(tlane + ((uint32_t)(16 * j) << 16), nacc, (er[j] >> 23) - 127, (ei[j] >> 23) - 127, ec.x, ec.y);
+                W[j] = read_rows<RG>(tlane + j * SUBC, nacc, split, (er[j] >> 23) - 127, (ei[j] >> 23) - 127, ec.x, ec.y);
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&T.tfree);
@@ -928,7 +978,7 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
                 if (fe[j] < 0) W[j] = make_float4(0.f, 0.f, 0.f, 0.f);
                 float4 q = cmul2(k, W[j]);
                 if (!bwd) q = add4(q, pre[j]);
-                publish(X + rn * A.slot_bytes + j * KGB, H + rn * A.hdr_words + j * NB * 4, q, ep.x, ep.y, u.tag + 1u);
+                publish(X + rn * A.slot_bytes + 4 * j * KGB, H + rn * A.hdr_words + 4 * j * NB * 4, q, ep.x, ep.y, u.tag + 1u);
             }
 #pragma unroll
         for (int j = 0; j < NRS; ++j) {
@@ -942,7 +992,7 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
 #pragma unroll
             for (int j = 0; j < NRS; ++j)
                 if (j ? fv1 : fv)
-                    __stcg(reinterpret_cast<uint4*>(X + (ri + NRING - 1 & NRING - 1) * A.slot_bytes + j * KGB),
+                    __stcg(reinterpret_cast<uint4*>(X + (ri + NRING - 1 & NRING - 1) * A.slot_bytes + 4 * j * KGB),
                            make_uint4(STALE, STALE, STALE, STALE));
             __syncwarp();
             ptx::fence_acq_rel_gpu();
@@ -976,7 +1026,7 @@ __device__ __forceinline__ int lines_end(Sm& T, int jo, int i) {
 template <int RG, int MT>
 __device__ __noinline__ bool run_general(const TeamArgs& A, Sm* Tp, Upd* up, int jo, int i) {
     Sm& T = *Tp;
-    constexpr int TBATCH = 512 / (NACC * 4 * RG);
+    constexpr int TBATCH = 512 / (MT / 64 * NACC * 4 * RG);
     const int lane = threadIdx.x & 31, c = lane & 3, rhs0 = 8 * (RG == 16 ? (int)(threadIdx.x >> 7) : 0) + 2 * c;
     const int B = T.B, cen = T.cen, team = T.team, nsol = T.nsol, U = T.U;
     const bool two = T.two;
@@ -1017,11 +1067,13 @@ __device__ __noinline__ bool run_general(const TeamArgs& A, Sm* Tp, Upd* up, int
             const int l0 = nkind == KIND_END ? (team ? T.N - A.g.b : A.g.b - 1) : wn.lo + wn.ia;
             // the coupled line of the next input
             const int l1 = (tn.bwd ? tn.role == ROLE_L : tn.role == ROLE_U) ? shapes[nkind].nl - 1 : 0;
-            publish_input<RG, MT>(A, Tp, jo, M, nkind, slot_of_solve(i + 1, nsol, cen, team), 0, u.tag + 1u, !tn.bwd, l0,
-                                  centre && two ? 0 : 2 + team, l1, -1, -1);
-            if (centre && two)                                  // and the upper front's first backward solve
+            // the centre also feeds the upper front's first backward solve: first, for the predicted scales may
+            // change once this rank's own input is out
+            if (centre && two)
                 publish_input<RG, MT>(A, Tp, jo, M, KIND_RING, slot_of_solve(U, 2 * U, cen, 1), 1,
                                       (unsigned)(jo * 2 * U + U) + 1u, false, T.win[cen + 1].lo + T.win[cen + 1].ia, 1, 0, -1, -1);
+            publish_input<RG, MT>(A, Tp, jo, M, nkind, slot_of_solve(i + 1, nsol, cen, team), 0, u.tag + 1u, !tn.bwd, l0,
+                                  centre && two ? 0 : 2 + team, l1, -1, -1);
         }
     }
     // as in run_lines
@@ -1041,7 +1093,8 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
     constexpr int KGB = 64 * RG;             // bytes of 8 published entries
     constexpr int GT = MT / 16;              // row groups of a tile
     constexpr int ACOLS = 4 * RG;            // columns of an accumulator: G times q's re hi, im hi, re lo, im lo
-    constexpr int TCOLS = NACC * ACOLS;      // accumulator columns of a tile
+    constexpr int NSUB = MT / 64;            // products of 4 row groups per tile and 16 input entries
+    constexpr int TCOLS = NSUB * NACC * ACOLS;   // accumulator columns of a tile
     constexpr int TBATCH = 512 / TCOLS;      // tiles with accumulators at a time
     const int B = A.g.B, N = A.g.N, cen = A.g.cen;
     const int two = A.T == 2;
@@ -1142,7 +1195,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                             // the tile's groups: at most two runs of stored groups (lane & 1: this lane's)
                             const int g0 = tl * GT, g1 = min(cs, g0 + GT);
                             const int m0 = max(0, min(g1, c0) - g0);
-                            const int run = lane & 1, h = lane >> 1;
+                            const int run = lane & 1;
                             const int cnt = run ? g1 - g0 - m0 : m0;
                             const int gr = run ? S.ng0 + S.a1 + max(0, g0 - c0) : S.a0 + g0;
                             const int kend = min(KP, k0 + A.KB);
@@ -1150,13 +1203,13 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                             for (int kc0 = k0; kc0 < kend; kc0 += TKC) {
                                 ok = wait_phase(&empty[stage], eph, limit, s_abort);
                                 if (!ok) break;
-                                const int kc = min(TKC, KP - kc0), per = 32 * kc;      // bytes of a group
+                                const int kc = min(TKC, KP - kc0), per = 32 * kc * A.halves;      // bytes of a group
                                 if (lane == 0)
-                                    ptx::mbar_expect_tx(&full[stage], (uint32_t)(A.halves * (g1 - g0) * per));
+                                    ptx::mbar_expect_tx(&full[stage], (uint32_t)((g1 - g0) * per));
                                 __syncwarp();
-                                if (lane < 2 * A.halves && cnt > 0)
-                                    ptx::bulk_g2s(ring + stage * A.stage_bytes + (h * GT + (run ? m0 : 0)) * per,
-                                                  base + ((size_t)kc0 * A.halves * ng + (size_t)kc * (h * ng + gr)) * 32,
+                                if (lane < 2 && cnt > 0)
+                                    ptx::bulk_g2s(ring + stage * A.stage_bytes + (run ? m0 : 0) * per,
+                                                  base + ((size_t)kc0 * ng + (size_t)kc * gr) * A.halves * 32,
                                                   (uint32_t)(cnt * per), &full[stage]);
                                 ++issued;
                                 if (++stage == A.stages) { stage = 0; eph ^= 1u; }
@@ -1179,74 +1232,75 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
         // the whole warp runs the loop: uniform operands, one elected lane issues; nothing is called
         // (after a call the compiler takes nothing for uniform), the gather warp makes the records
         const Shape* shapes = s_shape + 4;
-        const uint32_t idesc_all = ptx::umma_idesc_f16_bn(MT, 4 * RG), idesc_hi = ptx::umma_idesc_f16_bn(MT, 2 * RG);
+        const uint32_t idesc = ptx::umma_idesc_f16_bn(A.halves == 2 ? 128 : 64, 4 * RG);
         const uint64_t bdesc0 = ptx::umma_desc(ptx::smem_u32(Bbuf), KGB, 128u);
         const uint32_t a_s = ptx::smem_u32(ring);
-        const int split = A.halves == 2;
-        int stage = 0;
+        int stage = 0, seen = 0;                                  // seen: chunks ahead known to have landed
         uint32_t fph = 0, gph = 0, tph = 1, bph = 0;              // bph: a parity bit per part
         bool ok = true;
         for (int jo = 0; jo < nvis && ok; ++jo) {
 #pragma unroll 1
             for (int i = 0; i < nsol && ok; ++i) {
+                // the solve before has been read out of TMEM; operator chunks that have landed by then need no
+                // wait between the products
+                if (!(ok = wait_phase(tfree, tph, limit, s_abort))) break;
+                tph ^= 1u;
+#pragma unroll 1
+                for (; seen < A.stages; ++seen) {
+                    const int st = stage + seen, wrap = st >= A.stages;
+                    if (!__all_sync(0xffffffffu, ptx::mbar_try(&full[wrap ? st - A.stages : st], fph ^ (uint32_t)wrap))) break;
+                }
                 if (!(ok = wait_phase(bgo, gph, limit, s_abort))) break;    // of the solve's first gather
                 const Shape& S = shapes[kind_of(i, nsol, cen, team)];
                 const int KP = __shfl_sync(0xffffffffu, S.KP, 0), nt = __shfl_sync(0xffffffffu, S.nt, 0);
                 const int nch = __shfl_sync(0xffffffffu, S.nch, 0), nacc = __shfl_sync(0xffffffffu, S.nacc, 0);
 #pragma unroll 1
                 for (int tb = 0; (tb < nt || tb == 0) && ok; tb += TBATCH) {
-                    // the batch before has been read out of TMEM
-                    if (!(ok = wait_phase(tfree, tph, limit, s_abort))) break;
-                    tph ^= 1u;
-                    // an accumulator takes every nacc-th part of the chunks: it changes when rem overflows
+                    if (tb > 0) {                                 // so has the batch before
+                        if (!(ok = wait_phase(tfree, tph, limit, s_abort))) break;
+                        tph ^= 1u;
+                    }
 #pragma unroll 1
                     for (int k0 = 0; k0 < KP && ok; k0 += A.KB) {
-                        const int ke = min(KP, k0 + A.KB), n16 = (ke - k0) >> 4, part = (n16 + NBC - 1) / NBC;
+                        const int ke = min(KP, k0 + A.KB), part = 16 * gather_part((ke - k0) >> 4);
                         if (tb + k0 > 0 && !(ok = wait_phase(bgo, gph, limit, s_abort))) break;
                         gph ^= 1u;
-                        int have = 0, pj = 0;                     // gathered K = 16 steps, parts seen
 #pragma unroll 1
-                        for (int tl = tb; (tl < min(nt, tb + TBATCH) || have == 0) && ok; ++tl) {
-                            const bool real = tl < nt;            // a rank without rows only sees every part
-                            // chunk ch goes to accumulator ch nacc / nch
+                        for (int tl = tb; (tl < min(nt, tb + TBATCH) || tl == tb) && ok; ++tl) {
+                            // an accumulator takes a run of the chunks: chunk ch goes to accumulator ch nacc / nch
                             int ac = k0 / TKC * nacc, acc = 0;
                             while (ac >= nch) { ac -= nch; ++acc; }
                             int fresh = ac < nacc;                // the chunk is its accumulator's first
                             uint64_t bd = bdesc0;
 #pragma unroll 1
-                            for (int kc0 = k0; kc0 < ke; kc0 += TKC) {
-                                const int kc = min(TKC, KP - kc0), s1 = (kc0 - k0 + kc) >> 4;
-                                while (have < s1 && ok) {
-                                    ok = wait_phase(&bval[pj], bph >> pj & 1u, limit, s_abort);
+                            for (int kc0 = k0, pj = 0; kc0 < ke; ++pj) {
+                                if (tl == tb) {                   // the pass's first tile sees every part
+                                    if (!(ok = wait_phase(&bval[pj], bph >> pj & 1u, limit, s_abort))) break;
                                     bph ^= 1u << pj;
-                                    ++pj;
-                                    have = min(n16, have + part);
+                                }
+                                const int kpe = min(ke, kc0 + part);
+                                if (tl >= nt) kc0 = kpe;          // a rank without rows only sees them
+                                ptx::tc_fence_after();
+#pragma unroll 1
+                                for (; kc0 < kpe; kc0 += TKC) {
+                                    const int kc = min(TKC, KP - kc0);
+                                    if (--seen < 0) {
+                                        seen = 0;
+                                        if (!(ok = wait_phase(&full[stage], fph, limit, s_abort))) break;
+                                        ptx::tc_fence_after();
+                                    }
+                                    const uint32_t d = tmem + (uint32_t)((tl - tb) * TCOLS + acc * ACOLS);
+                                    const uint32_t ahi = a_s + (uint32_t)(stage * A.stage_bytes), sbo = (uint32_t)(kc * 16);
+                                    chunk_products<RG, NSUB>(d, ptx::umma_desc(ahi, 128u, sbo), 8 * A.halves * sbo / 16, bd, idesc,
+                                                             !fresh, kc);
+                                    bd += TKC / 16 * 2 * KGB / 16;
+                                    ptx::umma_commit_warp(&empty[stage]);
+                                    if (++stage == A.stages) { stage = 0; fph ^= 1u; }
+                                    ac += nacc;
+                                    fresh = ac >= nch;
+                                    if (fresh) { ac -= nch; ++acc; }
                                 }
                                 if (!ok) break;
-                                if (!real) continue;
-                                if (!(ok = wait_phase(&full[stage], fph, limit, s_abort))) break;
-                                ptx::tc_fence_after();
-                                const uint32_t d = tmem + (uint32_t)((tl - tb) * TCOLS + acc * ACOLS);
-                                uint32_t add = !fresh;
-                                const uint32_t ahi = a_s + (uint32_t)(stage * A.stage_bytes), sbo = (uint32_t)(kc * 16);
-                                uint64_t ah = ptx::umma_desc(ahi, 128u, sbo);
-                                uint64_t al = ptx::umma_desc(ahi + GT * 2 * sbo, 128u, sbo);
-#pragma unroll
-                                for (int ks = 0; ks < TKC / 16; ++ks) {
-                                    if (16 * ks < kc) {
-                                        ptx::umma_f16_warp(d, ah, bd, idesc_all, add);
-                                        if (split) ptx::umma_f16_warp(d + 2 * RG, al, bd, idesc_hi, 1u);
-                                        add = 1u;
-                                        ah += 16;                  // 256 bytes
-                                        al += 16;
-                                        bd += 2 * KGB / 16;
-                                    }
-                                }
-                                ptx::umma_commit_warp(&empty[stage]);
-                                if (++stage == A.stages) { stage = 0; fph ^= 1u; }
-                                ac += nacc;
-                                fresh = ac >= nch;
-                                if (fresh) { ac -= nch; ++acc; }
                             }
                         }
                         if (ok) ptx::umma_commit_warp(mdone);
@@ -1306,6 +1360,12 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                     if (!(ok = wait_phase(mdone, mph, limit, s_abort))) break;
                     mph ^= 1u;
                 }
+                // lane's part of the first gather: everything that does not need the headers before the poll
+                int kb = min(KP, A.KB), n16 = kb >> 4, part = gather_part(n16), my = lane * part;
+                uint32_t by = lane < NBC && my < n16 ? (uint32_t)(min(part, n16 - my) * 2 * KGB) : 0u;
+                unsigned char* dst = Bbuf + my * 2 * KGB;
+                const unsigned char* src = xs + (size_t)my * 2 * KGB;
+                if (by) ptx::mbar_expect_tx(&bfull[lane], by);
                 // poll the headers: max and used exponents of this lane's 4 right-hand sides
                 const int nv = ng8 * NB * 2;
                 unsigned mx0 = 0, mx1 = 0, mn0 = 0xffffffffu, mn1 = 0xffffffffu;
@@ -1337,28 +1397,38 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                     }
                 }
                 if (!ok) break;
+                // what the ranks cleared at the visit's beginning is seen by its gathers (once per visit; later
+                // clears are covered by the fence after each solve's headers)
+                if (kind == KIND_START) ptx::fence_acq_rel_gpu();
                 ptx::fence_proxy_async_global();
-                bool even = true;
+                if (by) ptx::bulk_g2s(dst, src, by, &bfull[lane]);
+                // each right-hand side has one scale in all headers: lane's columns are those of lane mod 2 NB
+                const unsigned x0 = __shfl_sync(0xffffffffu, mx0, lane & (2 * NB - 1));
+                const unsigned x1 = __shfl_sync(0xffffffffu, mx1, lane & (2 * NB - 1));
+                const bool none = lane >= nv;                         // fewer header words than lanes
+                const bool even = __all_sync(0xffffffffu, none || (((mx0 ^ mn0) | (mx1 ^ mn1) | (mx0 ^ x0) | (mx1 ^ x1)) &
+                                                                    0xff00ff00u) == 0u);
 #pragma unroll 1
                 for (int tb = 0; (tb < nt || tb == 0) && ok; tb += TBATCH)
 #pragma unroll 1
                     for (int k0 = 0; k0 < KP && ok; k0 += A.KB) {
-                        const int n16 = (min(KP, k0 + A.KB) - k0) >> 4, part = (n16 + NBC - 1) / NBC;
                         // the pass before has been multiplied
                         const bool first = tb == 0 && k0 == 0;
                         if (!first) {
                             if (!(ok = wait_phase(mdone, mph, limit, s_abort))) break;
                             mph ^= 1u;
+                            kb = min(KP, k0 + A.KB) - k0, n16 = kb >> 4, part = gather_part(n16), my = lane * part;
+                            by = lane < NBC && my < n16 ? (uint32_t)(min(part, n16 - my) * 2 * KGB) : 0u;
+                            if (by) {
+                                ptx::mbar_expect_tx(&bfull[lane], by);
+                                ptx::bulk_g2s(Bbuf + my * 2 * KGB, xs + (size_t)(k0 / 8 + my * 2) * KGB, by, &bfull[lane]);
+                            }
                         }
                         fresh = false;
-                        if (lane < NBC && lane * part < n16) {
-                            const uint32_t by = (uint32_t)(min(part, n16 - lane * part) * 2 * KGB);
-                            ptx::mbar_expect_tx(&bfull[lane], by);
-                            ptx::bulk_g2s(Bbuf + lane * part * 2 * KGB, xs + (size_t)(k0 / 8 + lane * part * 2) * KGB, by,
-                                          &bfull[lane]);
-                        }
                         for (int q = 0; q < NBC; ++q)
                             if (q * part < n16) lph ^= 1u << q;
+                        __syncwarp();
+                        if (even && lane == 0) ptx::mbar_arrive(bgo);
                         __syncwarp();
                         if (first) {
                             for (int s = 2 * NB; s < 32; s <<= 1) {
@@ -1367,11 +1437,6 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                                 mn0 = __vminu4(mn0, __shfl_xor_sync(0xffffffffu, mn0, s));
                                 mn1 = __vminu4(mn1, __shfl_xor_sync(0xffffffffu, mn1, s));
                             }
-                            even = __all_sync(0xffffffffu, (((mx0 ^ mn0) | (mx1 ^ mn1)) & 0xff00ff00u) == 0u);
-                        }
-                        if (even && lane == 0) ptx::mbar_arrive(bgo);
-                        __syncwarp();
-                        if (first) {
                             // scale exponents: of this input (the smallest used one), of the next
                             if (lane < 2 * NB) {
                                 float gn[4] = {0.f, 0.f, 0.f, 0.f};

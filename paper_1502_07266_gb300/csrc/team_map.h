@@ -119,17 +119,17 @@ __host__ __device__ __forceinline__ SolveGeo tm_geo(const AxisWin& wz, const Axi
 }
 
 // Stored tiles of one operator (FP16 forms): chunks of TKC input columns; in a
-// chunk of kc columns the hi parts of every row group (8 complex rows: 8 real
-// parts then 8 imaginary parts, each 8 rows x kc in K-major core matrices of
-// 8 x 16 bytes), then the lo parts.  A rank's groups are contiguous, so a chunk
-// of them is one copy for the hi and one for the lo parts.
+// chunk of kc columns every row group (8 complex rows) in turn: the hi parts of its
+// 8 real and of its 8 imaginary parts, then their lo parts, each 8 rows x kc in
+// K-major core matrices of 8 x 16 bytes.  A rank's groups are contiguous, so a chunk
+// of them is one copy.
 constexpr int TKC = 64;
 __host__ __device__ __forceinline__ int tm_kp(int K) { return 16 * tm_ceil(K, 16); }
 // byte offset of (chunk c, part h, group gr) and its size per group
 __host__ __device__ __forceinline__ size_t tm_tile(int c, int h, int gr, int ng, int KP, int halves, int* bytes) {
     const int kc = KP - c * TKC < TKC ? KP - c * TKC : TKC;
     *bytes = 2 * kc * 16;
-    return ((size_t)c * TKC * halves * ng + (size_t)kc * (h * ng + gr)) * 32;
+    return ((size_t)c * TKC * halves * ng + (size_t)kc * (gr * halves + h)) * 32;
 }
 __host__ __device__ __forceinline__ size_t tm_bytes(int ng, int KP, int halves) {
     return (size_t)ng * KP * halves * 32;
