@@ -316,6 +316,159 @@ k_dense_G(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __restric
     }
 }
 
+// The same for blocks of k <= KM: one thread per column.  With 64-row tiles a block
+// of 9 leaves six of seven rows and most of the scratch traffic to padding.  Here a
+// column's product input stays in its thread's shared slot and its k results in
+// registers, the factor block is read by broadcast (KM / 2 16-byte loads for 4 KM
+// fused multiply-adds), the columns share nothing else, and one barrier a step hands
+// over the next factor block.  The sums run in k_dense_G's order: the same bits.
+// Setup at n = 95, two fronts, b_aux = 2 (blocks of 9 to 25): 479 -> 173 ms.  What bounds it
+// then is the operator entries' way to memory and back (19.8 GB, 2.9 ms each) and the
+// steps' chain of shared-memory products.
+template <int KM>
+__global__ void __launch_bounds__(GW)
+k_dense_G_cols(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __restrict__ items, int nitems,
+               const float2* __restrict__ fac, long long off0, float2* __restrict__ Gt,
+               const long long* __restrict__ goff, float2* __restrict__ yscr, size_t yslot) {
+    __shared__ __align__(16) float2 Tt[2][KM * KM];   // [c][r]: two steps' factor blocks, transposed
+    __shared__ float2 W[KM][GW];                       // product input
+    __shared__ int so[KM], s_x[2];
+    const int jj = threadIdx.x;
+    const int N = g.N, m = (N - 1) / 2;
+    float2* Y = yscr + (size_t)blockIdx.x * yslot + jj;    // [N][KM][GW] forward values; x_m at block m
+
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+        const GItem I = items[it];
+        const DProb D = dp[I.p];
+        const Prob P = t.prob[D.fp];
+        const int k = P.k, Lz = P.Lz;
+        float2* Gp = Gt + goff[I.p];
+        const int jn = min(GW, D.n_in - I.j0);
+        int sa = -1, sx = -1;              // block row and x of the column's unit entry (-1: no column)
+        if (jj < jn) {
+            const int j = I.j0 + jj, per = D.in.nz * D.in.nl;
+            sx = j / per;
+            const int r = j - sx * per, l = r / D.in.nz;
+            sa = D.in.z0 + (r - l * D.in.nz) + Lz * (D.in.line0 + l - P.ylo);
+        }
+        __syncthreads();                   // previous item done with the shared arrays
+        if (jj == 0) s_x[0] = sx;
+        if (jj == jn - 1) s_x[1] = sx;
+        for (int a = jj; a < k; a += GW) {
+            const int lz = a % Lz, line = P.ylo + a / Lz;
+            int o = -1, base = 0;
+            for (int q = 0; q < D.nrect; ++q) {
+                const DRect R = D.out[q];
+                if (line >= R.line0 && line < R.line0 + R.nl && lz >= R.z0 && lz < R.z0 + R.nz)
+                    o = base + N * ((lz - R.z0) + R.nz * (line - R.line0));
+                base += R.nl * R.nz * N;
+            }
+            so[a] = o;
+        }
+        __syncthreads();
+        const int xa = s_x[0], xb = s_x[1];
+        const bool do_left = xa < m, do_right = xb > m;
+        const int nlf = do_left ? m - xa : 0, nrf = do_right ? xb - m : 0;
+        const int nsteps = nlf + nrf + N;
+        auto step_x = [&](int q) -> int {
+            if (q < nlf) return xa + q;
+            q -= nlf;
+            if (q < nrf) return xb - q;
+            q -= nrf;
+            if (q == 0) return m;
+            return q <= m ? m - q : q;
+        };
+        int i = step_x(0);
+        {
+            const float2* T0 = fac_block(fac, P, off0, i);
+            for (int e = jj; e < k * k; e += GW) {
+                const int r = e / k, c = e - r * k;
+                Tt[0][c * KM + r] = T0[(size_t)r * P.ldk + c];
+            }
+        }
+        for (int a = 0; a < k; ++a) W[a][jj] = make_float2(sx == i && sa == a ? 1.f : 0.f, 0.f);
+        __syncthreads();
+        for (int q = 0; q < nsteps; ++q) {
+            const bool more = q + 1 < nsteps;
+            const int inext = more ? step_x(q + 1) : -1;
+            constexpr int PF = (KM * KM + GW - 1) / GW;
+            float2 pf[PF];
+            if (more) {
+                const float2* Tn = fac_block(fac, P, off0, inext);
+#pragma unroll
+                for (int u = 0; u < PF; ++u) {
+                    const int e = jj + u * GW;
+                    pf[u] = make_float2(0.f, 0.f);
+                    if (e < k * k) pf[u] = Tn[(size_t)(e / k) * P.ldk + e % k];
+                }
+            }
+            float2 acc[KM];
+#pragma unroll
+            for (int a = 0; a < KM; ++a) acc[a] = make_float2(0.f, 0.f);
+#pragma unroll 1
+            for (int kk = 0; kk < k; ++kk) {
+                const float4* tr = reinterpret_cast<const float4*>(&Tt[q & 1][kk * KM]);
+                const float2 w = W[kk][jj];
+#pragma unroll
+                for (int a = 0; a < KM; a += 2) {
+                    const float4 v = tr[a / 2];
+                    cfma(acc[a], make_float2(v.x, v.y), w);
+                    cfma(acc[a + 1], make_float2(v.z, v.w), w);
+                }
+            }
+            if (more) {
+#pragma unroll
+                for (int u = 0; u < PF; ++u) {
+                    const int e = jj + u * GW;
+                    if (e < k * k) Tt[(q + 1) & 1][(e % k) * KM + e / k] = pf[u];
+                }
+            }
+            const bool fwd = q < nlf + nrf, mid = q == nlf + nrf;
+            const bool nfwd = q + 1 < nlf + nrf, nmid = q + 1 == nlf + nrf;
+            const bool has_y = i < m ? do_left && i >= xa : do_right && i <= xb;
+            const float2 cb = i < m ? t.c_up[i] : t.c_dn[i];                  // back substitution
+            const float2 cf = !more ? make_float2(0.f, 0.f) : (inext < m ? t.c_dn[inext] : t.c_up[inext]);
+            float2* Yi = Y + (size_t)i * KM * GW;
+#pragma unroll
+            for (int a = 0; a < KM; ++a) {
+                if (a >= k) break;
+                float2 val = acc[a];
+                if (fwd) {
+                    Yi[a * GW] = val;                                          // y_i
+                } else {
+                    if (mid) {
+                        Yi[a * GW] = val;                                      // x_m
+                    } else {
+                        // x_i = y_i - coupling * (T_i x_prev)
+                        const float2 yv = has_y ? Yi[a * GW] : make_float2(0.f, 0.f);
+                        val = csub(yv, cmul(cb, val));
+                    }
+                    const int o = so[a];
+                    if (o >= 0 && jj < jn) Gp[(size_t)(o + i) * D.n_in + I.j0 + jj] = val;
+                }
+                if (more) {
+                    const float2 e = make_float2(sx == inext && sa == a ? 1.f : 0.f, 0.f);
+                    float2 w;
+                    if (nfwd) {
+                        w = q + 1 == nlf ? e : csub(e, cmul(cf, val));         // a chain starts at its end block
+                    } else if (nmid) {
+                        w = e;
+                        if (do_left) w = csub(w, cmul(t.c_dn[m], Y[((size_t)(m - 1) * KM + a) * GW]));
+                        if (do_right) w = csub(w, cmul(t.c_up[m], Y[((size_t)(m + 1) * KM + a) * GW]));
+                    } else if (inext == m + 1) {
+                        w = Y[((size_t)m * KM + a) * GW];                      // the right back pass starts from x_m
+                    } else {
+                        w = val;
+                    }
+                    W[a][jj] = w;
+                }
+            }
+            i = inext;
+            __syncthreads();
+        }
+    }
+}
+
 // Pack one output tile (operator p, 64 complex rows) into the apply's format.
 struct PItem { int p, mt; };
 
@@ -1175,6 +1328,21 @@ static void build_dense_table(helm_ctx* h, const std::vector<AxisWin>& win, int 
     *gbytes = off;
 }
 
+// Kernels of the operator columns by block size: one thread per column up to k = 32,
+// where its k results fit in registers (166 of them at 32); 64-row tiles beyond, which they
+// fill by more than half.  Setup at n = 95 with blocks of 9 to 25: 173 ms against 479 ms
+// with 64-row tiles throughout.
+typedef void (*GCols)(Geom, Tables, const DProb*, const GItem*, int, const float2*, long long, float2*, const long long*,
+                      float2*, size_t);
+struct GClass { int km; GCols fn; };
+const GClass G_COLS[] = {{10, k_dense_G_cols<10>}, {16, k_dense_G_cols<16>}, {26, k_dense_G_cols<26>}, {32, k_dense_G_cols<32>}};
+constexpr int GCLASSES = sizeof(G_COLS) / sizeof(G_COLS[0]) + 1;
+int g_class(int k) {
+    int q = 0;
+    while (q < GCLASSES - 1 && k > G_COLS[q].km) ++q;
+    return q;
+}
+
 // Factors and restricted operators of slabs Ma..Mb, for the line blocks
 // Pa..Pb (and the first block's backward operator when Pa = 0): the build of
 // helm_setup (all of them) and of helm_update_velocity (those a box touches).
@@ -1245,7 +1413,7 @@ static int dense_build(helm_ctx* h, const Prob* prob, int Ma, int Mb, int Pa, in
         }
         DTRY(launch_factor_range(h, M0 * B, (M1 - M0) * B, fac, off0, HELM_FP32, st));
         // work items and temporary operator offsets of the chunk
-        std::vector<GItem> items;
+        std::vector<GItem> items, by_class[GCLASSES];
         std::vector<PItem> pitems;
         std::vector<int> ops;
         long long go = 0;
@@ -1257,13 +1425,14 @@ static int dense_build(helm_ctx* h, const Prob* prob, int Ma, int Mb, int Pa, in
                 if (dp[p].n_out == 0) continue;
                 goff[p] = go;
                 go += (long long)dp[p].n_out * dp[p].n_in;
-                for (int j0 = 0; j0 < dp[p].n_in; j0 += GW) items.push_back(GItem{p, j0});
+                for (int j0 = 0; j0 < dp[p].n_in; j0 += GW) by_class[g_class(prob[dp[p].fp].k)].push_back(GItem{p, j0});
                 if (h->opts.precision == HELM_FP32)
                     for (int mt = 0; mt < dp[p].n_mt; ++mt) pitems.push_back(PItem{p, mt});
                 else
                     ops.push_back(p);
             }
         }
+        for (const std::vector<GItem>& v : by_class) items.insert(items.end(), v.begin(), v.end());
         if (items.size() > items_cap) {
             if (d_items) cudaFree(d_items);
             d_items = nullptr;
@@ -1280,11 +1449,26 @@ static int dense_build(helm_ctx* h, const Prob* prob, int Ma, int Mb, int Pa, in
         if (!pitems.empty())
             DTRY(cudaMemcpyAsync(d_pitems, pitems.data(), pitems.size() * sizeof(PItem), cudaMemcpyHostToDevice, st));
         DTRY(cudaMemcpyAsync(d_goff, goff.data(), sizeof(long long) * P, cudaMemcpyHostToDevice, st));
-        const int nblk = (int)std::min<size_t>(items.size(), (size_t)gblocks);
-        k_dense_G<<<nblk, GT, gsm, st>>>(h->g, h->t, h->dprob, d_items, (int)items.size(), fac, off0, Gt, d_goff,
-                                         yscr, yslot);
-        h->launches++;
-        DTRY(cudaGetLastError());
+        size_t first = 0;
+        for (int q = 0; q < GCLASSES; ++q) {
+            const size_t n = by_class[q].size();
+            if (n == 0) continue;
+            const GItem* it = d_items + first;
+            first += n;
+            if (q == GCLASSES - 1) {
+                k_dense_G<<<(int)std::min<size_t>(n, (size_t)gblocks), GT, gsm, st>>>(
+                    h->g, h->t, h->dprob, it, (int)n, fac, off0, Gt, d_goff, yscr, yslot);
+            } else {
+                // as many blocks as fit on the chip and the forward values' scratch holds
+                int occ = 1;
+                DTRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, G_COLS[q].fn, GW, 0));
+                const size_t slot = (size_t)N * G_COLS[q].km * GW;
+                const size_t blk = std::min(std::min(n, (size_t)nsm * std::max(occ, 1)), gblocks * yslot / slot);
+                G_COLS[q].fn<<<(int)blk, GW, 0, st>>>(h->g, h->t, h->dprob, it, (int)n, fac, off0, Gt, d_goff, yscr, slot);
+            }
+            h->launches++;
+            DTRY(cudaGetLastError());
+        }
         if (h->opts.precision == HELM_FP32) {
             k_dense_pack<<<(int)pitems.size(), 256, 0, st>>>(h->dprob, d_pitems, Gt, d_goff, h->dG);
             h->launches++;
