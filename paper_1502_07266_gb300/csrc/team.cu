@@ -223,7 +223,7 @@ constexpr int MMA_WARP = 8, RING_WARP = 9, GATHER_WARP = 10;
 constexpr int TT = 32 * 11;                 // threads of a CTA
 constexpr int MAXST = 16;                   // most ring stages
 constexpr int NBC = 2;                      // parts a gather is split into
-constexpr int NACC = 2;                     // accumulators of a tile, over runs of input chunks
+constexpr int NACC = 4;                     // accumulators of a tile, over runs of input chunks
 constexpr unsigned STALE = 0xffffffffu;     // a word not published yet (no pair of converted FP16 values has it)
 constexpr long long TEAM_WAIT = 4000000000ll;   // about 2 s at 2 GHz
 
@@ -279,53 +279,41 @@ __device__ __forceinline__ int gather_part(int n16) {
     return (n16 + NBC * U - 1) / (NBC * U) * U;
 }
 
-// Y = G q of one row pair of right-hand sides from a tile's accumulators: in
-// each, the row's real parts (lane t/4) and imaginary parts (lane t/4 + 8) times
-// q's re hi, im hi, re lo, im lo; with split operators the products of their lo
-// parts with q's hi parts 16 lanes further on.  The accumulators cover successive
-// runs of input chunks and are added here in rounded FP32 (the tensor core's own
-// additions do not round to nearest: one long chain costs accuracy).  er, ei:
-// exponents of the row's scales; c0, c1: of the columns'.
+// One accumulator of a row pair of right-hand sides, added to R and I: the row's
+// real parts (lane t/4) and imaginary parts (lane t/4 + 8) times q's re hi, im hi,
+// re lo, im lo; with split operators the products of their lo parts with q's hi
+// parts 16 lanes further on.  The accumulators cover successive runs of input
+// chunks and are added here in rounded FP32: the tensor core's own additions do not
+// round to nearest, and the error of an apply grows with their chain (n = 31, one
+// front: 8.4e-6 with 2 accumulators, 6.5e-6 with 4).
 template <int RG>
-__device__ __forceinline__ float4 read_rows(uint32_t ta, int nacc, bool split, int er, int ei, int c0, int c1) {
-    float R[4] = {0.f, 0.f, 0.f, 0.f}, I[4] = {0.f, 0.f, 0.f, 0.f};
+__device__ __forceinline__ void add_rows(uint32_t ta, bool split, float (&R)[4], float (&I)[4]) {
+    float rh[4], mh[4], rl[4], ml[4], lr[4] = {0.f, 0.f, 0.f, 0.f}, lm[4] = {0.f, 0.f, 0.f, 0.f};
     __syncwarp();                                    // the TMEM loads are warp-collective
-    float rh[NACC][4], mh[NACC][4], rl[NACC][4], ml[NACC][4], lr[NACC][4], lm[NACC][4];
-#pragma unroll
-    for (int a = 0; a < NACC; ++a)
-        if (a < nacc) {
-            ptx::tmem_ld16x8(ta + a * 4 * RG, rh[a]);
-            ptx::tmem_ld16x8(ta + a * 4 * RG + RG, mh[a]);
-            ptx::tmem_ld16x8(ta + a * 4 * RG + 2 * RG, rl[a]);
-            ptx::tmem_ld16x8(ta + a * 4 * RG + 3 * RG, ml[a]);
-            if (split) {
-                ptx::tmem_ld16x8(ta + (16u << 16) + a * 4 * RG, lr[a]);
-                ptx::tmem_ld16x8(ta + (16u << 16) + a * 4 * RG + RG, lm[a]);
-            }
-        }
+    ptx::tmem_ld16x8(ta, rh);
+    ptx::tmem_ld16x8(ta + RG, mh);
+    ptx::tmem_ld16x8(ta + 2 * RG, rl);
+    ptx::tmem_ld16x8(ta + 3 * RG, ml);
+    if (split) {
+        ptx::tmem_ld16x8(ta + (16u << 16), lr);
+        ptx::tmem_ld16x8(ta + (16u << 16) + RG, lm);
+    }
     ptx::tmem_wait_ld();
+    ptx::reg_tie4(rh);
+    ptx::reg_tie4(mh);
+    ptx::reg_tie4(rl);
+    ptx::reg_tie4(ml);
+    ptx::reg_tie4(lr);
+    ptx::reg_tie4(lm);
 #pragma unroll
-    for (int a = 0; a < NACC; ++a)
-        if (a < nacc) {
-            ptx::reg_tie4(rh[a]);
-            ptx::reg_tie4(mh[a]);
-            ptx::reg_tie4(rl[a]);
-            ptx::reg_tie4(ml[a]);
-            if (split) {
-                ptx::reg_tie4(lr[a]);
-                ptx::reg_tie4(lm[a]);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    rl[a][q] += lr[a][q];
-                    ml[a][q] += lm[a][q];
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                R[q] += rh[a][q] + rl[a][q];
-                I[q] += mh[a][q] + ml[a][q];
-            }
-        }
+    for (int q = 0; q < 4; ++q) {
+        R[q] += rh[q] + (rl[q] + lr[q]);
+        I[q] += mh[q] + (ml[q] + lm[q]);
+    }
+}
+
+// Y = G q from the sums.  er, ei: exponents of the row's scales; c0, c1: of the columns'.
+__device__ __forceinline__ float4 scale_rows(const float (&R)[4], const float (&I)[4], int er, int ei, int c0, int c1) {
     const int a0 = -(er + c0), a1 = -(er + c1), b0 = -(ei + c0), b1 = -(ei + c1);
     const int lo = min(min(a0, a1), min(b0, b1)), hi = max(max(a0, a1), max(b0, b1));
     if (__any_sync(0xffffffffu, lo < -126 || hi > 127))          // far from one: in two steps
@@ -430,6 +418,7 @@ struct Sm {
     uint64_t bgo;                // a gather pass may be multiplied
     uint64_t eready;             // its scale exponents are in shared memory
     uint64_t mdone;              // its products are complete
+    uint64_t sacc[NACC - 1];     // an accumulator's products are complete (one tile; otherwise with sdone)
     uint64_t sdone;              // a tile batch's products are complete
     uint64_t tfree;              // its accumulators have been read (CW arrivals)
     uint64_t cbar;               // barrier of the update warps (CW arrivals)
@@ -456,7 +445,7 @@ struct Sm {
 
 // An update warp's place in the barriers' phases.
 struct Upd {
-    uint32_t sph, cph, xph, vph; // vph: a parity bit per gathered part
+    uint32_t sph, cph, xph, vph; // vph: a parity bit per gathered part; sph: per accumulator, the last for sdone
     unsigned arrivals, tag;      // tag: number of the solve, from 1
 };
 
@@ -672,9 +661,11 @@ __device__ __noinline__ void general_rows(const TeamArgs& A, Sm* T, int M, int i
             const int r = 8 * gid + ii;
             const int nl = rect ? g.out1.nl : g.out0.nl, nz = rect ? g.out1.nz : g.out0.nz;
             const float* sc = A.scale + soff + (long long)((rect ? S.ng0 : 0) + gid) * 16 + ii;
-            float4 X = read_rows<RG>(tlane + (uint32_t)(j * SUBC + (tl - tb) * TCOLS), S.nacc, A.halves == 2,
-                                     (__float_as_int(__ldg(sc)) >> 23) - 127,
-                                     (__float_as_int(__ldg(sc + 8)) >> 23) - 127, ec0, ec1);
+            float R[4] = {0.f, 0.f, 0.f, 0.f}, I[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int a = 0; a < S.nacc; ++a)
+                add_rows<RG>(tlane + (uint32_t)(j * SUBC + (tl - tb) * TCOLS + a * 4 * RG), A.halves == 2, R, I);
+            float4 X = scale_rows(R, I, (__float_as_int(__ldg(sc)) >> 23) - 127, (__float_as_int(__ldg(sc + 8)) >> 23) - 127,
+                                  ec0, ec1);
             if (r < (rect ? g.n1 : g.n0)) {
                 const int l = r % nl, tt = r / nl, x = tt / nz;
                 const int lz = (rect ? g.out1.z0 : g.out0.z0) + tt - x * nz;
@@ -788,6 +779,14 @@ __device__ __forceinline__ bool validate(Sm& T, Upd& u, const unsigned char* xs,
         }
     }
     return ok;
+}
+
+// Waits until accumulator a of nacc has all its products.
+__device__ __forceinline__ bool wait_acc(Sm& T, Upd& u, int a, int nacc, long long limit) {
+    const int b = a == nacc - 1 ? NACC - 1 : a;
+    const bool r = wait_phase(b == NACC - 1 ? &T.sdone : &T.sacc[b], u.sph >> b & 1u, limit, &T.abort);
+    u.sph ^= 1u << b;
+    return r;
 }
 
 // Barrier of the update warps.
@@ -957,16 +956,23 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
         ok = validate<RG>(T, u, T.X + ri * A.slot_bytes, KP, A.KB, T.limit);
         if (ok) ok = wait_phase(&T.eready, u.xph, T.limit, &T.abort);
         u.xph ^= 1u;
-        if (ok) ok = wait_phase(&T.sdone, u.sph, T.limit, &T.abort);
-        u.sph ^= 1u;
         if (!ok) break;
-        ptx::tc_fence_after();
         const int2 ec = *reinterpret_cast<const int2*>(&T.ecol[rhs0]), ep = *reinterpret_cast<const int2*>(&T.epred[rhs0]);
+        // accumulators are read as they complete, while the next one is multiplied
+        float R[NRS][4] = {}, I[NRS][4] = {};
+#pragma unroll 1
+        for (int a = 0; a < nacc && ok; ++a) {
+            if (!(ok = wait_acc(T, u, a, nacc, T.limit))) break;
+            ptx::tc_fence_after();
+#pragma unroll
+            for (int j = 0; j < NRS; ++j)
+                if (j ? fv1 : fv) add_rows<RG>(tlane + j * SUBC + a * 4 * RG, split, R[j], I[j]);
+        }
+        if (!ok) break;
         float4 W[NRS];
 #pragma unroll
         for (int j = 0; j < NRS; ++j)
-            if (j ? fv1 : fv)
-                W[j] = read_rows<RG>(tlane + j * SUBC, nacc, split, (er[j] >> 23) - 127, (ei[j] >> 23) - 127, ec.x, ec.y);
+            if (j ? fv1 : fv) W[j] = scale_rows(R[j], I[j], (er[j] >> 23) - 127, (ei[j] >> 23) - 127, ec.x, ec.y);
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&T.tfree);
@@ -1049,8 +1055,7 @@ __device__ __noinline__ bool run_general(const TeamArgs& A, Sm* Tp, Upd* up, int
             if (ok) ok = wait_phase(&T.eready, u.xph, limit, &T.abort);
             u.xph ^= 1u;
         }
-        if (ok) ok = wait_phase(&T.sdone, u.sph, limit, &T.abort);
-        u.sph ^= 1u;
+        for (int a = 0; a < S.nacc && ok; ++a) ok = wait_acc(T, u, a, S.nacc, limit);
         if (!ok) break;
         ptx::tc_fence_after();
         general_rows<RG, MT>(A, Tp, M, i, tb, T.soff[op_slot(t.Mp, t.bwd, B)], T.tslot, T.ecol[rhs0], T.ecol[rhs0 + 1]);
@@ -1132,6 +1137,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
         ptx::mbar_init(eready, 1);
         ptx::mbar_init(mdone, 1);
         ptx::mbar_init(sdone, 1);
+        for (int q = 0; q < NACC - 1; ++q) ptx::mbar_init(&S_.sacc[q], 1);
         ptx::mbar_init(tfree, CW);
         ptx::mbar_init(&S_.cbar, CW);
         ptx::mbar_init(&S_.xbar, 1);
@@ -1298,14 +1304,22 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                                     if (++stage == A.stages) { stage = 0; fph ^= 1u; }
                                     ac += nacc;
                                     fresh = ac >= nch;
-                                    if (fresh) { ac -= nch; ++acc; }
+                                    if (fresh) {
+                                        if (nt == 1 && acc < nacc - 1) ptx::umma_commit_warp(&S_.sacc[acc]);
+                                        ac -= nch;
+                                        ++acc;
+                                    }
                                 }
                                 if (!ok) break;
                             }
                         }
                         if (ok) ptx::umma_commit_warp(mdone);
                     }
-                    if (ok) ptx::umma_commit_warp(sdone);
+                    if (ok) {
+                        if (nt != 1)
+                            for (int q = 0; q < nacc - 1; ++q) ptx::umma_commit_warp(&S_.sacc[q]);
+                        ptx::umma_commit_warp(sdone);
+                    }
                 }
             }
         }
