@@ -587,8 +587,8 @@ def run_gpu(args):
     if args.form == "dense":
         nsolves, alg_bytes, macs = _dense_model(wl.n, wl.b, wl.d, DENSE_ENTRY_BYTES[args.precision],
                                                 args.schedule, args.b_aux)
-        kernel = {"fp32": "k_dense<FP32 SIMT>", "split_fp16": "k_dense<FP16 hi+lo, tcgen05>",
-                  "fp16": "k_dense<FP16 hi, tcgen05>"}[args.precision]
+        kernel = {"fp32": "k_dense<FP32 SIMT>", "split_fp16": "k_team<FP16 hi+lo, tcgen05>",
+                  "fp16": "k_team<FP16 hi, tcgen05>"}[args.precision]
         traffic = _dense_traffic(wl.n, args.precision, args.schedule, args.b_aux)
         chain = {"dependent_solves_per_apply": nsolves, "us_per_solve": per_launch_ms * 1e3 / nsolves}
         flops = 8.0 * macs * R
