@@ -38,16 +38,6 @@ __device__ __forceinline__ bool mbar_try_cluster(uint64_t* bar, uint32_t parity)
                  : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
     return ok != 0;
 }
-// Up to n polls of a phase in a tight loop; the barrier by its shared address.
-__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, uint32_t n) {
-    uint32_t ok;
-    asm volatile("{\n .reg .pred p, q;\n .reg .u32 i;\n mov.u32 i, %3;\n"
-                 "POLL_LOOP_%=:\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                 " @p bra POLL_DONE_%=;\n sub.u32 i, i, 1;\n setp.ne.u32 q, i, 0;\n @q bra POLL_LOOP_%=;\n"
-                 "POLL_DONE_%=:\n selp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(n) : "memory");
-    return ok != 0;
-}
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -67,18 +57,12 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
 __device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
-// ---- asynchronous copies global -> shared (per thread, 4 or 8 bytes) -------
+// ---- asynchronous copies global -> shared (per thread, 8 bytes) ------------
 // Not ordered by bar.sync: the issuing thread waits with cp_async_wait_all.
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
@@ -94,11 +78,6 @@ __device__ __forceinline__ uint32_t mapa(const void* local, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(smem_u32(local)), "r"(rank));
     return out;
 }
-__device__ __forceinline__ float ld_dsmem_f32(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
 __device__ __forceinline__ float2 ld_dsmem_f32x2(uint32_t addr) {
     float2 v;
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
@@ -110,7 +89,6 @@ __device__ __forceinline__ float4 ld_dsmem_f32x4(uint32_t addr) {
                  : "r"(addr) : "memory");
     return v;
 }
-__device__ __forceinline__ void fence_acq_rel_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 
 // ---- global-memory flags ----------------------------------------------------
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
@@ -189,14 +167,8 @@ __host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N) {
 // bytes (8 N values); the descriptor's LBO then steps 8 K rows and its SBO 8 N
 // columns.
 __host__ __device__ constexpr uint32_t umma_idesc_f16_bn(int M, int N) { return umma_idesc_f16(M, N) | (1u << 16); }
-// D[tmem] (+)= A[smem] * B[smem]^T, issued by one thread.
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// The same two from a converged warp: one lane is elected to issue, and with
+// D[tmem] (+)= A[smem] * B[smem]^T, and an arrival on bar when every product issued
+// so far has completed, from a converged warp: one lane is elected to issue, and with
 // operands equal in every lane the compiler keeps them in uniform registers
 // (about 30 cycles per product instead of 70 to 250 from a divergent branch).
 __device__ __forceinline__ void umma_f16_warp(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
@@ -210,27 +182,6 @@ __device__ __forceinline__ void umma_commit_warp(uint64_t* bar) {
                  " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}"
                  ::"r"(smem_u32(bar)) : "memory");
 }
-// Arrive once on `bar` when every MMA this thread issued so far has completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 ::"r"(smem_u32(bar)) : "memory");
-}
-// 32 lanes x 8 consecutive 32-bit columns: thread i of the warp gets lane
-// (base lane + i), columns col..col+7.  The values are valid after tmem_wait8.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-                 : "r"(taddr) : "memory");
-}
-// 32 lanes x 16 consecutive 32-bit columns (valid after tmem_wait_ld + reg_tie16).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
-                 "%13, %14, %15}, [%16];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
-                   "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]),
-                   "=f"(v[15])
-                 : "r"(taddr) : "memory");
-}
 // 16 lanes x 8 consecutive 32-bit columns spread over the warp: thread t gets
 // lane t/4, columns 2 (t mod 4) and + 1 in v[0], v[1], and lane t/4 + 8 in v[2],
 // v[3] (valid after tmem_wait_ld + reg_tie4).
@@ -241,17 +192,9 @@ __device__ __forceinline__ void tmem_ld16x8(uint32_t taddr, float (&v)[4]) {
 __device__ __forceinline__ void reg_tie4(float (&v)[4]) {
     asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]));
 }
+// Then reg_tie4: every use of v depends on that statement, so none is scheduled
+// before the wait (volatile statements keep their order).
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// Placed after tmem_wait_ld (volatile statements keep their order): every use
-// of v depends on this statement, so none is scheduled before the wait.
-__device__ __forceinline__ void reg_tie8(float (&v)[8]) {
-    asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]));
-}
-__device__ __forceinline__ void reg_tie16(float (&v)[16]) {
-    asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
-                      "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]),
-                      "+f"(v[15]));
-}
 // Waits for the warp's outstanding TMEM loads; the registers are tied to the
 // wait so that no use is scheduled before it.
 __device__ __forceinline__ void tmem_wait8(float (&a)[8], float (&b)[8]) {
