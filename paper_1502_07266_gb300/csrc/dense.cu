@@ -60,6 +60,19 @@ __device__ __forceinline__ void cfma(float2& acc, float2 a, float2 b) {
     acc.y = fmaf(a.y, b.x, acc.y);
 }
 
+// y - c v, the coupling step of the substitutions, with every rounding written out:
+// left to the compiler it contracts to other multiply-adds in k_dense_G than in
+// k_dense_G_cols, and operators that differ in their last bit differ by a whole
+// FP16 step here and there once they are rounded to FP16.  FIRST says which product
+// of the real part is rounded before the other is added to it.
+enum { FIRST_YY = 0, FIRST_XX = 1 };
+__device__ __forceinline__ float2 sub_coupled(float2 y, float2 c, float2 v, int first) {
+    const float re = first == FIRST_XX ? __fmaf_rn(-c.y, v.y, __fmul_rn(c.x, v.x))
+                                       : __fmaf_rn(c.x, v.x, -__fmul_rn(c.y, v.y));
+    const float im = __fmaf_rn(c.y, v.x, __fmul_rn(c.x, v.y));
+    return make_float2(__fsub_rn(y.x, re), __fsub_rn(y.y, im));
+}
+
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 // Bytes per K column of the main part of one stored tile (FP32 form): 64 complex
@@ -269,7 +282,7 @@ k_dense_G(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __restric
                         // back substitution: x_i = y_i - coupling * (T_i x_prev)
                         const float2 cp = (i < m) ? t.c_up[i] : t.c_dn[i];
                         const float2 yv = has_y(i) ? *ys : make_float2(0.f, 0.f);
-                        val = csub(yv, cmul(cp, val));
+                        val = sub_coupled(yv, cp, val, !has_y(i) && i < m ? FIRST_XX : FIRST_YY);
                     }
                     if (!fwd) {                                  // val = x_i: output rows
                         if (mid) Xm[a * GW + jj] = val;
@@ -296,12 +309,12 @@ k_dense_G(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __restric
                                 w = e;
                             } else {
                                 const float2 cp = (inext < m) ? t.c_dn[inext] : t.c_up[inext];
-                                w = csub(e, cmul(cp, acc[qq][cc]));
+                                w = sub_coupled(e, cp, acc[qq][cc], FIRST_XX);
                             }
                         } else if (nmid) {
                             w = e;
-                            if (do_left) w = csub(w, cmul(t.c_dn[m], Y[((size_t)(m - 1) * 64 + a) * GW + jj]));
-                            if (do_right) w = csub(w, cmul(t.c_up[m], Y[((size_t)(m + 1) * 64 + a) * GW + jj]));
+                            if (do_left) w = sub_coupled(w, t.c_dn[m], Y[((size_t)(m - 1) * 64 + a) * GW + jj], FIRST_XX);
+                            if (do_right) w = sub_coupled(w, t.c_up[m], Y[((size_t)(m + 1) * 64 + a) * GW + jj], FIRST_XX);
                         } else if (inext == m + 1) {
                             w = Xm[a * GW + jj];                 // the right back pass starts from x_m
                         } else {
@@ -321,7 +334,8 @@ k_dense_G(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __restric
 // column's product input stays in its thread's shared slot and its k results in
 // registers, the factor block is read by broadcast (KM / 2 16-byte loads for 4 KM
 // fused multiply-adds), the columns share nothing else, and one barrier a step hands
-// over the next factor block.  The sums run in k_dense_G's order: the same bits.
+// over the next factor block.  The sums run in k_dense_G's order and round as there:
+// the same bits.
 // Setup at n = 95, two fronts, b_aux = 2 (blocks of 9 to 25): 479 -> 173 ms.  What bounds it
 // then is the operator entries' way to memory and back (19.8 GB, 2.9 ms each) and the
 // steps' chain of shared-memory products.
@@ -441,7 +455,7 @@ k_dense_G_cols(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __re
                     } else {
                         // x_i = y_i - coupling * (T_i x_prev)
                         const float2 yv = has_y ? Yi[a * GW] : make_float2(0.f, 0.f);
-                        val = csub(yv, cmul(cb, val));
+                        val = sub_coupled(yv, cb, val, !has_y && i < m ? FIRST_XX : FIRST_YY);
                     }
                     const int o = so[a];
                     if (o >= 0 && jj < jn) Gp[(size_t)(o + i) * D.n_in + I.j0 + jj] = val;
@@ -450,11 +464,11 @@ k_dense_G_cols(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __re
                     const float2 e = make_float2(sx == inext && sa == a ? 1.f : 0.f, 0.f);
                     float2 w;
                     if (nfwd) {
-                        w = q + 1 == nlf ? e : csub(e, cmul(cf, val));         // a chain starts at its end block
+                        w = q + 1 == nlf ? e : sub_coupled(e, cf, val, FIRST_XX);         // a chain starts at its end block
                     } else if (nmid) {
                         w = e;
-                        if (do_left) w = csub(w, cmul(t.c_dn[m], Y[((size_t)(m - 1) * KM + a) * GW]));
-                        if (do_right) w = csub(w, cmul(t.c_up[m], Y[((size_t)(m + 1) * KM + a) * GW]));
+                        if (do_left) w = sub_coupled(w, t.c_dn[m], Y[((size_t)(m - 1) * KM + a) * GW], FIRST_XX);
+                        if (do_right) w = sub_coupled(w, t.c_up[m], Y[((size_t)(m + 1) * KM + a) * GW], FIRST_XX);
                     } else if (inext == m + 1) {
                         w = Y[((size_t)m * KM + a) * GW];                      // the right back pass starts from x_m
                     } else {
