@@ -35,13 +35,11 @@
 // header of the 8 entries; a gather that finds unequal scales brings them to the
 // smallest in shared memory before the product.
 //
-// Headers carry the solve's number and are stored after the parts, but no fence
-// orders the two (one costs 1.2 k cycles after a store, once a solve on the
-// critical path): a slot's words are all ones before they are published, no pair
-// of converted FP16 values is (a NaN converts to 0x7fff), and a gather that still finds such a word fetches it
-// again until it is there.  For that a slot is cleared by the ranks that filled it,
-// one ring solve after its own (every rank has read it by then), off the critical
-// path, and used again three ring solves later.
+// Headers carry the solve's number and are released at GPU scope after the parts; the
+// gathering warp reads them until they are all there, fences (acquire, and a proxy
+// fence, for bulk copies are another proxy), and only then copies the parts.  A slot is written again NRING ring solves later: whoever does that
+// has read headers of the solves between, which their ranks stored after they had
+// multiplied, hence gathered, the slot's input.
 //
 // Per CTA: eight warps apply the updates, one warp issues the products, one
 // streams the operator through a ring, one polls headers and gathers.  The loops
@@ -224,7 +222,6 @@ constexpr int TT = 32 * 11;                 // threads of a CTA
 constexpr int MAXST = 16;                   // most ring stages
 constexpr int NBC = 2;                      // parts a gather is split into
 constexpr int NACC = 4;                     // accumulators of a tile, over runs of input chunks
-constexpr unsigned STALE = 0xffffffffu;     // a word not published yet (no pair of converted FP16 values has it)
 constexpr long long TEAM_WAIT = 4000000000ll;   // about 2 s at 2 GHz
 
 struct TeamArgs {
@@ -414,7 +411,6 @@ struct Sm {
     uint64_t full[MAXST];        // operator chunk landed
     uint64_t empty[MAXST];       // operator chunk consumed
     uint64_t bfull[NBC];         // part of the gather landed
-    uint64_t bval[NBC];          // and every word of it is current (CW arrivals)
     uint64_t bgo;                // a gather pass may be multiplied
     uint64_t eready;             // its scale exponents are in shared memory
     uint64_t mdone;              // its products are complete
@@ -445,11 +441,11 @@ struct Sm {
 
 // An update warp's place in the barriers' phases.
 struct Upd {
-    uint32_t sph, cph, xph, vph; // vph: a parity bit per gathered part; sph: per accumulator, the last for sdone
+    uint32_t sph, cph, xph;      // sph: a parity bit per accumulator, the last for sdone
     unsigned arrivals, tag;      // tag: number of the solve, from 1
 };
 
-// The warp that publishes (and clears) group gi of the rank, right-hand sides
+// The warp that publishes group gi of the rank, right-hand sides
 // 8 pcb ..: the one whose accumulator rows they are in a one-tile solve, so that an
 // entry's words stay with one warp.
 template <int RG, int MT>
@@ -468,11 +464,11 @@ __device__ __forceinline__ void fail(const TeamArgs& A, Sm& S) {
     S.abort = 1;
 }
 
-// Publishes one row's value for two right-hand sides: FP16 hi and lo parts, scaled
-// by 2^e0 and 2^e1.  The four lanes of a row trade their words so that each stores
-// one part of the row for 8 right-hand sides (16 bytes, at p); lanes 0..3 store the
-// header words of the 8 entries at hd.
-__device__ __forceinline__ void publish(unsigned char* p, u64* hd, float4 v, int e0, int e1, unsigned tag) {
+// Stores one row's value for two right-hand sides: FP16 hi and lo parts, scaled by
+// 2^e0 and 2^e1.  The four lanes of a row trade their words so that each stores one
+// part of the row for 8 right-hand sides (16 bytes, at p).  Returns the value half of
+// the lane's header word (lanes 0..3: those of the 8 entries).
+__device__ __forceinline__ unsigned store_parts(unsigned char* p, float4 v, int e0, int e1) {
     const int lane = threadIdx.x & 31;
     unsigned m = max(__float_as_uint(fabsf(v.x)), __float_as_uint(fabsf(v.y))) >> 23 |
                  max(__float_as_uint(fabsf(v.z)), __float_as_uint(fabsf(v.w))) >> 23 << 16;
@@ -493,22 +489,19 @@ __device__ __forceinline__ void publish(unsigned char* p, u64* hd, float4 v, int
     const unsigned px = c0 ? r0 : w0, py = c0 ? w1 : r0, qx = c0 ? r1 : w2, qy = c0 ? w3 : r1;
     const unsigned rx = __shfl_xor_sync(0xffffffffu, c1 ? px : qx, 2), ry = __shfl_xor_sync(0xffffffffu, c1 ? py : qy, 2);
     __stcg(reinterpret_cast<uint4*>(p), make_uint4(c1 ? rx : px, c1 ? ry : py, c1 ? qx : rx, c1 ? qy : ry));
-    if (lane < 4)
-        ptx::st_relaxed_gpu_u64(hd + lane, (u64)tag << 32 | (unsigned)(f0 | (e0 + 128) << 8 | f1 << 16 | (e1 + 128) << 24));
+    return (unsigned)(f0 | (e0 + 128) << 8 | f1 << 16 | (e1 + 128) << 24);
 }
-
-// Marks the rank's entries of a slot as not published.
-template <int RG, int MT>
-__device__ __noinline__ void clear_slot(unsigned char* xs, int kg0, int kg1) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int STEP = RG == 8 && MT == 128 ? 8 : 4;        // groups between a warp's own (warp_of)
-    const int pcb = RG == 16 ? warp >> 2 : 0;
-    const int gi = RG == 8 && MT == 64 && warp > 3 ? kg1 - kg0 : warp & (STEP - 1);
-#pragma unroll 4
-    for (int kg = kg0 + gi; kg < kg1; kg += STEP)
-        __stcg(reinterpret_cast<uint4*>(xs + (size_t)kg * 64 * RG + part_offset<RG>(pcb, lane)),
-               make_uint4(STALE, STALE, STALE, STALE));
-    __syncwarp();
+// The header words of a warp's parts, after a __syncwarp that orders the other lanes'
+// parts before: released, or relaxed behind the warp's own release fence.  One apply,
+// two fronts, n = 127 with 64 right-hand sides: 182 ms with releasing stores, 190 ms
+// with a release fence, 207 ms with acquire-release fences here and at the gather.
+__device__ __forceinline__ void release_header(u64* hd, unsigned w, unsigned tag) {
+    const int lane = threadIdx.x & 31;
+    if (lane < 4) ptx::st_release_gpu_u64(hd + lane, (u64)tag << 32 | w);
+}
+__device__ __forceinline__ void store_header(u64* hd, unsigned w, unsigned tag) {
+    const int lane = threadIdx.x & 31;
+    if (lane < 4) ptx::st_relaxed_gpu_u64(hd + lane, (u64)tag << 32 | w);
 }
 
 // Boundary of slab visits jo-1 and jo (Algorithm 6).
@@ -698,6 +691,10 @@ __device__ __noinline__ void publish_input(const TeamArgs& A, Sm* T, int jo, int
     const float2 *b1 = T->Qf + max(q1, 0) * VL, *b2 = T->Qf + max(q2, 0) * VL;
     unsigned char* xs = T->X + up * T->Xteam + slot * A.slot_bytes;
     u64* hd = T->H + up * T->Hteam + (size_t)slot * A.hdr_words;
+    constexpr int PB = 4;                    // groups of 8 entries a warp stores under one fence
+    unsigned hw[PB];
+    u64* hp[PB];
+    int held = 0;
 #pragma unroll 1
     for (int t = 0; t < (S.kg1 - S.kg0) * NB; ++t) {
         const int gi = t / NB, pcb = t % NB, kg = S.kg0 + gi;
@@ -724,61 +721,28 @@ __device__ __noinline__ void publish_input(const TeamArgs& A, Sm* T, int jo, int
             if (l == l1) v = add4(v, __ldcg(reinterpret_cast<const float4*>(b1 + eo)));
             if (l == l2) v = add4(v, __ldcg(reinterpret_cast<const float4*>(b2 + eo)));
         }
-        publish(xs + (size_t)kg * KGB + part_offset<RG>(pcb, lane), hd + (kg * NB + pcb) * 4, v, e0, e1, tag);
-    }
-}
-
-// The gathered parts as they land: words that are not there yet are fetched until
-// they are (the headers are stored after the parts, but nothing orders the two on
-// their way).
-template <int RG>
-__device__ __forceinline__ bool validate(Sm& T, Upd& u, const unsigned char* xs, int KP, int KB, long long limit) {
-    constexpr int KGB = 64 * RG;
-    const int tid = threadIdx.x, lane = tid & 31;
-    bool ok = true;
-#pragma unroll 1
-    for (int k0 = 0; k0 < KP && ok; k0 += KB) {
-        const int n16 = (min(KP, k0 + KB) - k0) >> 4, part = gather_part(n16);
-        const int vpart = part * (2 * KGB / 16);
-        int left = n16 * (2 * KGB / 16), base = 0;
-#pragma unroll 1
-        for (int q = 0; q < NBC && left > 0; ++q) {
-            if (!(ok = wait_phase(&T.bfull[q], u.vph >> q & 1u, limit, &T.abort))) break;
-            u.vph ^= 1u << q;
-            const int nvec = min(vpart, left);
-            uint4* b = reinterpret_cast<uint4*>(T.Bbuf) + base;
-            int good = 1, wrote = 0;
-#pragma unroll 1
-            for (int v0 = tid; v0 < nvec; v0 += 8 * 32 * CW) {
-                unsigned m = 0u;
+        const unsigned w = store_parts(xs + (size_t)kg * KGB + part_offset<RG>(pcb, lane), v, e0, e1);
 #pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    const uint4 w = b[min(v0 + r * 32 * CW, nvec - 1)];
-                    m = max(m, max(max(w.x, w.y), max(w.z, w.w)));
-                }
-                if (m == STALE) {
-#pragma unroll 1
-                    for (int v = v0; v < min(nvec, v0 + 8 * 32 * CW); v += 32 * CW) {
-                        const uint4* src = reinterpret_cast<const uint4*>(xs + (size_t)k0 * (KGB / 8)) + base + v;
-                        const long long t0 = clock64();
-                        uint4 x = b[v];
-                        while (good && max(max(x.x, x.y), max(x.z, x.w)) == STALE) {
-                            x = ptx::ld_relaxed_gpu_v4(src);
-                            b[v] = x;
-                            wrote = 1;
-                            good = clock64() - t0 <= limit && !T.abort;
-                        }
-                    }
-                }
+        for (int q = 0; q < PB; ++q)
+            if (q == held) {
+                hw[q] = w;
+                hp[q] = hd + (kg * NB + pcb) * 4;
             }
-            if (wrote) ptx::fence_proxy_async_smem();
-            if (!(ok = __all_sync(0xffffffffu, good))) break;
-            if (lane == 0) ptx::mbar_arrive(&T.bval[q]);
-            base += vpart;
-            left -= vpart;
+        if (++held == PB) {
+            __syncwarp();
+            ptx::fence_release_gpu();
+#pragma unroll
+            for (int q = 0; q < PB; ++q) store_header(hp[q], hw[q], tag);
+            held = 0;
         }
     }
-    return ok;
+    if (held > 0) {
+        __syncwarp();
+        ptx::fence_release_gpu();
+#pragma unroll
+        for (int q = 0; q < PB; ++q)
+            if (q < held) store_header(hp[q], hw[q], tag);
+    }
 }
 
 // Waits until accumulator a of nacc has all its products.
@@ -840,24 +804,15 @@ __device__ __forceinline__ int kind_of_slot(int sl) {
 }
 __device__ __forceinline__ int tail_groups(const Shape& S) { return S.KP / 8 - ((S.K + 7) >> 3); }   // 0 or 1
 
-// A visit's beginning: the slots of the visit before are cleared, its result and
-// the new right-hand side pass through z, the records are made, and (after the
-// group's barrier) the first input is published.
+// A visit's beginning: the result of the visit before and the new right-hand side pass
+// through z, the records are made, the entries that pad an input are set to zero, and
+// (after the group's barrier) the first input is published.
 template <int RG, int MT>
 __device__ __noinline__ bool begin_visit(const TeamArgs& A, Sm* Tp, Upd* up, int jo) {
     Sm& T = *Tp;
     const int B = T.B, cen = T.cen, team = T.team, nsol = T.nsol;
     const int tid = threadIdx.x;
     Shape* shapes = T.shape + 8;
-    const unsigned slots = used_slots(nsol, cen, team);
-    const bool tail = T.rank == T.C - 1;               // this rank's are the entries that pad an input
-    if (jo > 0) {
-#pragma unroll 1
-        for (int sl = 0; sl <= SLOT_START; ++sl) {
-            const Shape& S = shapes[kind_of_slot(sl)];
-            if (slots >> sl & 1u) clear_slot<RG, MT>(T.X + sl * A.slot_bytes, S.kg0, S.kg1 + (tail ? tail_groups(S) : 0));
-        }
-    }
     boundary_phase<RG>(A, Tp, jo);
     if (jo == 2 * B - 1) return true;
     const int M = pass_pos(jo, B, cen).M;
@@ -865,17 +820,21 @@ __device__ __noinline__ bool begin_visit(const TeamArgs& A, Sm* Tp, Upd* up, int
     Upd u = *up;
     bool ok = cta_sync(T, u, T.limit);                 // everybody is done with the records of the visit before
     *up = u;
-    if (tid < 32) make_shapes(shapes, T.win, T.N, B, cen, T.two, team, M, T.rank, T.C, MT / 16, tid & 31);
+    if (tid < 32) {
+        make_shapes(shapes, T.win, T.N, B, cen, T.two, team, M, T.rank, T.C, MT / 16, tid & 31);
+        // the entries that pad an input are the last rank's, zero for the whole visit
+        const unsigned slots = T.rank == T.C - 1 ? used_slots(nsol, cen, team) : 0u;
+#pragma unroll 1
+        for (int sl = 0; sl <= SLOT_START; ++sl) {
+            const Shape& S = shapes[kind_of_slot(sl)];
+            if ((slots >> sl & 1u) && tail_groups(S))
+                for (int q = tid; q < 4 * RG; q += 32)
+                    __stcg(reinterpret_cast<uint4*>(T.X + sl * A.slot_bytes + (size_t)S.kg1 * 64 * RG) + q,
+                           make_uint4(0u, 0u, 0u, 0u));
+        }
+    }
     ok = ok && group_sync(A, Tp, up);
     if (!ok) return false;
-    if (tail)
-#pragma unroll 1
-        for (int sl = 0; sl <= SLOT_START; ++sl) {     // zero for the whole visit
-            const Shape& S = shapes[kind_of_slot(sl)];
-            if ((slots >> sl & 1u) && tail_groups(S) && tid < 4 * RG)
-                __stcg(reinterpret_cast<uint4*>(T.X + sl * A.slot_bytes + (size_t)S.kg1 * 64 * RG) + tid,
-                       make_uint4(0u, 0u, 0u, 0u));
-        }
     const AxisWin& w0 = T.win[tm_solve(0, B, cen, team).Mp];
     publish_input<RG, MT>(A, Tp, jo, M, KIND_START, SLOT_START, 0, up->tag + 1u, true, w0.lo + w0.ia, -1, -1, -1, -1);
     return true;
@@ -931,7 +890,6 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
     const float* scale = A.scale + cg0 * 16 + ii;
     const int nacc = min(NACC, tm_ceil(KP, TKC));
     int ri = slot_of_solve(i, nsol, cen, team);           // ring slot of solve i
-    bool after = ring_before(i, cen, team) > 0;           // a ring solve precedes it
     Upd u = *up;
     bool ok = true;
 #pragma unroll 1
@@ -953,8 +911,7 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
             if (o >= 0) pre[j] = ptx::ld_cg_f32x4_here((bwd ? line : gl) + o);
         }
         const float2 k = make_float2(fs * pc->x, fs * pc->y);
-        ok = validate<RG>(T, u, T.X + ri * A.slot_bytes, KP, A.KB, T.limit);
-        if (ok) ok = wait_phase(&T.eready, u.xph, T.limit, &T.abort);
+        ok = wait_phase(&T.eready, u.xph, T.limit, &T.abort);
         u.xph ^= 1u;
         if (!ok) break;
         const int2 ec = *reinterpret_cast<const int2*>(&T.ecol[rhs0]), ep = *reinterpret_cast<const int2*>(&T.epred[rhs0]);
@@ -976,6 +933,7 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&T.tfree);
+        unsigned hw[NRS];
         const int rn = i + 1 == nsol - 1 ? SLOT_END : (!team && i + 1 == cen ? SLOT_CENTRE : (ri + 1) & (NRING - 1));
 #pragma unroll
         for (int j = 0; j < NRS; ++j)
@@ -984,26 +942,17 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
                 if (fe[j] < 0) W[j] = make_float4(0.f, 0.f, 0.f, 0.f);
                 float4 q = cmul2(k, W[j]);
                 if (!bwd) q = add4(q, pre[j]);
-                publish(X + rn * A.slot_bytes + 4 * j * KGB, H + rn * A.hdr_words + 4 * j * NB * 4, q, ep.x, ep.y, u.tag + 1u);
+                hw[j] = store_parts(X + rn * A.slot_bytes + 4 * j * KGB, q, ep.x, ep.y);
             }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < NRS; ++j)
+            if (j ? fv1 : fv) release_header(H + rn * A.hdr_words + 4 * j * NB * 4, hw[j], u.tag + 1u);
 #pragma unroll
         for (int j = 0; j < NRS; ++j) {
             const int o = bwd ? fz[j] : fe[j];
             if (o >= 0) *reinterpret_cast<float4*>((bwd ? zl : line) + o) = W[j];
         }
-        // Every rank has read the ring's input before this one (each published this one after it): its
-        // words become stale for the input three solves on.  The fence orders that before this warp's
-        // next headers; a gather sees it after it has seen those.
-        if (after) {
-#pragma unroll
-            for (int j = 0; j < NRS; ++j)
-                if (j ? fv1 : fv)
-                    __stcg(reinterpret_cast<uint4*>(X + (ri + NRING - 1 & NRING - 1) * A.slot_bytes + 4 * j * KGB),
-                           make_uint4(STALE, STALE, STALE, STALE));
-            __syncwarp();
-            ptx::fence_acq_rel_gpu();
-        }
-        after = true;
         ri = rn & (NRING - 1);
         pc += dy;
         po += dy;
@@ -1042,7 +991,6 @@ __device__ __noinline__ bool run_general(const TeamArgs& A, Sm* Tp, Upd* up, int
     const TeamSolve t = tm_solve(i, B, cen, team);
     const int kind = kind_of(i, nsol, cen, team);
     const Shape& S = shapes[kind];
-    const int slot = slot_of_solve(i, nsol, cen, team);
     const bool more = i + 1 < nsol, centre = kind == KIND_CENTRE;
     const bool into_centre = two && !t.bwd && (team ? i == U - 1 : i == cen - 1);
     Upd u = *up;
@@ -1050,9 +998,8 @@ __device__ __noinline__ bool run_general(const TeamArgs& A, Sm* Tp, Upd* up, int
     bool ok = true;
 #pragma unroll 1
     for (int tb = 0; (tb < S.nt || tb == 0) && ok; tb += TBATCH) {
-        ok = validate<RG>(T, u, T.X + slot * A.slot_bytes, S.KP, A.KB, limit);
         if (tb == 0) {
-            if (ok) ok = wait_phase(&T.eready, u.xph, limit, &T.abort);
+            ok = wait_phase(&T.eready, u.xph, limit, &T.abort);
             u.xph ^= 1u;
         }
         for (int a = 0; a < S.nacc && ok; ++a) ok = wait_acc(T, u, a, S.nacc, limit);
@@ -1081,12 +1028,6 @@ __device__ __noinline__ bool run_general(const TeamArgs& A, Sm* Tp, Upd* up, int
                                   centre && two ? 0 : 2 + team, l1, -1, -1);
         }
     }
-    // as in run_lines
-    const int ip = ring_before(i, cen, team);
-    if (ok && kind == KIND_RING && ip > 0) {
-        clear_slot<RG, MT>(T.X + slot_of_solve(ip, nsol, cen, team) * A.slot_bytes, S.kg0, S.kg1);
-        ptx::fence_acq_rel_gpu();
-    }
     *up = u;
     return ok;
 }
@@ -1111,7 +1052,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
     long long* s_soff = reinterpret_cast<long long*>(s_cup + N); // [B + 2]
     long long* s_off = s_soff + B + 2;                           // [B + 2]
     AxisWin* s_win = reinterpret_cast<AxisWin*>(s_off + B + 2);  // [B]
-    uint64_t *full = S_.full, *empty = S_.empty, *bfull = S_.bfull, *bval = S_.bval;
+    uint64_t *full = S_.full, *empty = S_.empty, *bfull = S_.bfull;
     uint64_t *bgo = &S_.bgo, *eready = &S_.eready, *mdone = &S_.mdone, *sdone = &S_.sdone, *tfree = &S_.tfree;
     volatile int* s_abort = &S_.abort;
     Shape* s_shape = S_.shape;
@@ -1129,10 +1070,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
             ptx::mbar_init(&full[q], 1);
             ptx::mbar_init(&empty[q], 1);
         }
-        for (int q = 0; q < NBC; ++q) {
-            ptx::mbar_init(&bfull[q], 1);
-            ptx::mbar_init(&bval[q], CW);
-        }
+        for (int q = 0; q < NBC; ++q) ptx::mbar_init(&bfull[q], 1);
         ptx::mbar_init(bgo, 1);
         ptx::mbar_init(eready, 1);
         ptx::mbar_init(mdone, 1);
@@ -1281,7 +1219,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
 #pragma unroll 1
                             for (int kc0 = k0, pj = 0; kc0 < ke; ++pj) {
                                 if (tl == tb) {                   // the pass's first tile sees every part
-                                    if (!(ok = wait_phase(&bval[pj], bph >> pj & 1u, limit, s_abort))) break;
+                                    if (!(ok = wait_phase(&bfull[pj], bph >> pj & 1u, limit, s_abort))) break;
                                     bph ^= 1u << pj;
                                 }
                                 const int kpe = min(ke, kc0 + part);
@@ -1358,7 +1296,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                                                    : (kind == KIND_START ? SLOT_START : (kind == KIND_END ? SLOT_END : SLOT_CENTRE));
                 const unsigned char* xs = S_.X + slot * A.slot_bytes;
                 const u64* hw0 = S_.H + slot * A.hdr_words;
-                const uint4* hd = reinterpret_cast<const uint4*>(hw0) + lane;
+                const u64* hd = hw0 + 2 * lane;
                 // the lines the slab's right-hand side enters the next input on
                 int gl0 = 0, gln = 0;
                 if (i + 1 < nsol) {
@@ -1386,7 +1324,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                 const long long t0 = clock64();
 #pragma unroll 1
                 for (int v0 = 0; v0 < nv && ok; v0 += 32 * 8) {
-                    uint4 w[8];
+                    ulonglong2 w[8];
                     unsigned pend = 0;
 #pragma unroll
                     for (int u = 0; u < 8; ++u)
@@ -1394,15 +1332,15 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                     while (__any_sync(0xffffffffu, pend != 0)) {
 #pragma unroll
                         for (int u = 0; u < 8; ++u)
-                            if (pend >> u & 1) w[u] = ptx::ld_relaxed_gpu_v4(hd + v0 + 32 * u);
+                            if (pend >> u & 1) w[u] = ptx::ld_relaxed_gpu_v2u64(hd + 2 * (v0 + 32 * u));
 #pragma unroll
                         for (int u = 0; u < 8; ++u)
-                            if ((pend >> u & 1) && w[u].y == tag && w[u].w == tag) {
+                            if ((pend >> u & 1) && (unsigned)(w[u].x >> 32) == tag && (unsigned)(w[u].y >> 32) == tag) {
                                 pend &= ~(1u << u);
-                                mx0 = __vmaxu4(mx0, w[u].x);
-                                mx1 = __vmaxu4(mx1, w[u].z);
-                                mn0 = __vminu4(mn0, w[u].x);
-                                mn1 = __vminu4(mn1, w[u].z);
+                                mx0 = __vmaxu4(mx0, (unsigned)w[u].x);
+                                mx1 = __vmaxu4(mx1, (unsigned)w[u].y);
+                                mn0 = __vminu4(mn0, (unsigned)w[u].x);
+                                mn1 = __vminu4(mn1, (unsigned)w[u].y);
                             }
                         if (__any_sync(0xffffffffu, pend != 0 && (clock64() - t0 > limit || *s_abort))) {
                             ok = false;
@@ -1411,9 +1349,10 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                     }
                 }
                 if (!ok) break;
-                // what the ranks cleared at the visit's beginning is seen by its gathers (once per visit; later
-                // clears are covered by the fence after each solve's headers)
-                if (kind == KIND_START) ptx::fence_acq_rel_gpu();
+                // every lane has read headers released after their parts: its fence, then the warp's barrier, order
+                // the parts before the copies of lanes 0 and 1
+                ptx::fence_acquire_gpu();
+                __syncwarp();
                 ptx::fence_proxy_async_global();
                 if (by) ptx::bulk_g2s(dst, src, by, &bfull[lane]);
                 // each right-hand side has one scale in all headers: lane's columns are those of lane mod 2 NB
@@ -1474,13 +1413,11 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                             }
                             __syncwarp();
                             if (lane == 0) ptx::mbar_arrive(eready);
-                            // what the ranks cleared before they published this input is seen by the next gathers
-                            ptx::fence_acq_rel_gpu();
                         }
                         if (!even) {
                             // unequal scales: bring every group of 8 entries to the smallest exponent
                             for (int q = 0; q < NBC && ok; ++q)
-                                if (q * part < n16) ok = wait_phase(&bval[q], ~(lph >> q) & 1u, limit, s_abort);
+                                if (q * part < n16) ok = wait_phase(&bfull[q], ~(lph >> q) & 1u, limit, s_abort);
                             if (!ok) break;
 #pragma unroll 1
                             for (int v = lane; v < n16 * 2 * 4 * NB * 8; v += 32) {
@@ -1516,7 +1453,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
         }
     } else {
         // ------------------------------------------------------ update warps
-        Upd u = {0, 0, 0, 0, 0, 0};
+        Upd u = {0, 0, 0, 0, 0};
         bool ok = true;
 #pragma unroll 1
         for (int jo = 0; jo <= nvis && ok; ++jo) {
@@ -1809,9 +1746,8 @@ cudaError_t launch_team_apply(helm_ctx* h, const float2* r, float2* z, int nrhs,
         A.off_misc = P.off_misc;
         A.wait_cycles = h->opts.wait_cycles;
         A.unmet = h->opts.debug_unmet_wait;
-        // nothing published, no header of this launch, empty tables and counters
-        cudaError_t e = cudaMemsetAsync(work + P.oX, 0xff, (P.oH - P.oX) * sizeof(float2), st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(work + P.oH, 0, (P.total - P.oH) * sizeof(float2), st);
+        // no header of this launch, empty tables and counters
+        cudaError_t e = cudaMemsetAsync(work + P.oH, 0, (P.total - P.oH) * sizeof(float2), st);
         if (e != cudaSuccess) return e;
         // the CTAs wait on one another: a cooperative launch starts them together or not at all
         cudaLaunchConfig_t cfg;

@@ -54,8 +54,8 @@ __host__ __device__ __forceinline__ TeamSolve tm_solve(int i, int B, int c, int 
 }
 
 // Slots of published inputs: a ring for the solves of a visit, one each for the
-// centre, the last solve and the first.  A ring slot is cleared in the ring solve
-// after its own (every rank has read it by then) and used again three later.
+// centre, the last solve and the first.  A slot's next input comes at least two
+// solves later, when every rank has read the one before.
 constexpr int NRING = 4, SLOT_CENTRE = NRING, SLOT_END = NRING + 1, SLOT_START = NRING + 2;
 __host__ __device__ __forceinline__ int slot_of_solve(int i, int nsol, int cen, int upper) {
     if (i == 0) return SLOT_START;
@@ -64,11 +64,6 @@ __host__ __device__ __forceinline__ int slot_of_solve(int i, int nsol, int cen, 
     if (i == cen) return SLOT_CENTRE;
     return (i < cen ? i - 1 : i - 2) & (NRING - 1);
 }
-// The ring solve before ring solve i (0: none).
-__host__ __device__ __forceinline__ int ring_before(int i, int cen, int upper) {
-    return !upper && i - 1 == cen ? i - 2 : i - 1;
-}
-
 // Index sets of solve (slab window wz, line block window wy) of a team.  A
 // boundary line block (0, and B-1 with two fronts) takes its own entries forward
 // and feeds the one line next to its neighbour; backward it takes that line.

@@ -116,3 +116,33 @@ def test_repeated_applies_are_the_same_bits(helm):
         assert torch.equal(S.apply(ft), z)
     assert S.status() == helm.HELM_OK
     S.close()
+
+
+@pytest.mark.parametrize("n,b,d,b_aux,schedule,nrhs,clusters,precision", [
+    (14, 3, 2, 2, "two_front", 33, 0, "split_fp16"),    # two lines a block
+    (13, 4, 2, 3, "one_front", 9, 0, "fp16"),
+    (15, 4, 3, 2, "two_front", 5, 0, "split_fp16"),     # three, of which 8 is no multiple
+    (33, 6, 2, 6, "one_front", 17, 1, "split_fp16"),    # inputs of several gathers, several tiles a rank
+    (33, 6, 2, 6, "one_front", 3, 2, "fp16"),
+    (16, 3, 1, 2, "two_front", 9, 1, "split_fp16"),     # one line a block, several tiles a rank
+])
+def test_every_path_repeats_its_bits(helm, n, b, d, b_aux, schedule, nrhs, clusters, precision):
+    """20 applies of unequal sources give the same bits, and they are those of the FP32
+    form up to the two forms' bounds (1e-5 each; 3e-3 with FP16 operators)."""
+    om = W.omega_for(n)
+    c = torch.from_numpy(W.velocity_random(n, b, seed=n).astype(np.float32)).cuda()
+    f = W.random_rhs(nrhs, n, b, seed=8).astype(np.complex64)
+    f *= np.exp(np.linspace(-4.0, 4.0, f.shape[2], dtype=np.float32))[None, None, :, None]
+    ft = torch.from_numpy(f).cuda()
+    S = helm.Solver(c, om, n, b, d, b_aux=b_aux, precision=precision, apply_form="dense", schedule=schedule,
+                    dense_clusters=clusters)
+    z = S.apply(ft).clone()
+    for _ in range(19):
+        assert torch.equal(S.apply(ft), z)
+    assert S.status() == helm.HELM_OK
+    S.close()
+    S = helm.Solver(c, om, n, b, d, b_aux=b_aux, precision="fp32", apply_form="dense", schedule=schedule)
+    w = S.apply(ft)
+    S.close()
+    err = torch.linalg.vector_norm((z - w).reshape(nrhs, -1), dim=1) / torch.linalg.vector_norm(w.reshape(nrhs, -1), dim=1)
+    assert float(err.max()) <= (2e-5 if precision == "split_fp16" else 3e-3 + 1e-5), err
