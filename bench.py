@@ -402,22 +402,26 @@ def _dense_setup_model(n: int, b: int, d: int, schedule: str = "one_front", b_au
 
 
 DENSE_ENTRY_BYTES = {"fp32": 8, "split_fp16": 8, "fp16": 4}
+# the files the dense apply kernel of a precision is compiled from
+DENSE_SOURCES = {"fp32": ("dense.cu", "dense_sched.h", "ptx.cuh"),
+                 "fp16": ("team.cu", "team_map.h", "dense_sched.h", "ptx.cuh")}
 
 
 def _dense_traffic(n: int, precision: str, schedule: str, b_aux: int):
     """DRAM bytes per dense apply launch from the committed ncu summary, if it
-    was taken on the current kernel source and the same schedule (else None)."""
+    was taken on the current source of that precision's kernel and the same
+    schedule (else None)."""
     path = os.path.join(ROOT, "profiles", "dense_traffic.txt")
     csrc = os.path.join(ROOT, "paper_1502_07266_gb300", "csrc")
+    sources = DENSE_SOURCES["fp32" if precision == "fp32" else "fp16"]
     try:
-        digest = hashlib.sha1(open(os.path.join(csrc, "dense.cu"), "rb").read()).hexdigest()
-        digest_s = hashlib.sha1(open(os.path.join(csrc, "dense_sched.h"), "rb").read()).hexdigest()
+        digest = {f: hashlib.sha1(open(os.path.join(csrc, f), "rb").read()).hexdigest() for f in sources}
         fields = {}
         for line in open(path):
             if ":" in line:
                 key, val = line.split(":", 1)
                 fields[key.strip()] = val.strip()
-        if (fields.get("dense.cu sha1") != digest or fields.get("dense_sched.h sha1") != digest_s
+        if (any(fields.get(f + " sha1") != digest[f] for f in sources)
                 or fields.get("precision") != precision
                 or fields.get("schedule") != schedule or int(fields.get("b_aux", -1)) != (b_aux or 6)):
             return None
