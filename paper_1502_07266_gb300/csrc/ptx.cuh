@@ -110,6 +110,11 @@ __device__ __forceinline__ ulonglong2 ld_relaxed_gpu_v2u64(const void* p) {
 __device__ __forceinline__ void st_relaxed_gpu_u64(unsigned long long* p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+// Two FP32 additions, each rounded to nearest, in one instruction: a[0..1] += b[0..1].
+__device__ __forceinline__ void add2(float* a, const float* b) {
+    asm("{\n .reg .b64 x, y;\n mov.b64 x, {%0, %1};\n mov.b64 y, {%2, %3};\n add.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;\n}"
+        : "+f"(a[0]), "+f"(a[1]) : "f"(b[0]), "f"(b[1]));
+}
 // Loads that stay where they are written (volatile): prefetches into registers
 // ahead of a wait.
 __device__ __forceinline__ float4 ld_cg_f32x4_here(const void* p) {
@@ -185,12 +190,22 @@ __device__ __forceinline__ void umma_commit_warp(uint64_t* bar) {
                  " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}"
                  ::"r"(smem_u32(bar)) : "memory");
 }
-// 16 lanes x 8 consecutive 32-bit columns spread over the warp: thread t gets
-// lane t/4, columns 2 (t mod 4) and + 1 in v[0], v[1], and lane t/4 + 8 in v[2],
-// v[3] (valid after tmem_wait_ld + reg_tie4).
-__device__ __forceinline__ void tmem_ld16x8(uint32_t taddr, float (&v)[4]) {
-    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(taddr) : "memory");
+// 16 lanes x 32 (or 16) consecutive 32-bit columns spread over the warp: of column
+// block q of 8, thread t gets lane t/4, columns 2 (t mod 4) and + 1 in v[q][0], v[q][1],
+// and lane t/4 + 8 in v[q][2], v[q][3] (valid after tmem_wait_ld + reg_tie4).
+__device__ __forceinline__ void tmem_ld16x32(uint32_t taddr, float (&v)[4][4]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+                 "%14, %15}, [%16];"
+                 : "=f"(v[0][0]), "=f"(v[0][1]), "=f"(v[0][2]), "=f"(v[0][3]), "=f"(v[1][0]), "=f"(v[1][1]),
+                   "=f"(v[1][2]), "=f"(v[1][3]), "=f"(v[2][0]), "=f"(v[2][1]), "=f"(v[2][2]), "=f"(v[2][3]),
+                   "=f"(v[3][0]), "=f"(v[3][1]), "=f"(v[3][2]), "=f"(v[3][3])
+                 : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16x16(uint32_t taddr, float (&v)[2][4]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0][0]), "=f"(v[0][1]), "=f"(v[0][2]), "=f"(v[0][3]), "=f"(v[1][0]), "=f"(v[1][1]),
+                   "=f"(v[1][2]), "=f"(v[1][3])
+                 : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void reg_tie4(float (&v)[4]) {
     asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]));

@@ -221,7 +221,9 @@ constexpr int MMA_WARP = 8, RING_WARP = 9, GATHER_WARP = 10;
 constexpr int TT = 32 * 11;                 // threads of a CTA
 constexpr int MAXST = 16;                   // most ring stages
 constexpr int NBC = 2;                      // parts a gather is split into
-constexpr int NACC = 4;                     // accumulators of a tile, over runs of input chunks
+// Accumulators of a tile in TMEM: its 512 columns over products of 64 rows by 4 RG columns
+// (more than 8 would only stretch the read-out).
+__host__ __device__ constexpr int acc_slots(int RG, int MT) { return RG == 16 && MT == 128 ? 4 : 8; }
 constexpr long long TEAM_WAIT = 4000000000ll;   // about 2 s at 2 GHz
 
 struct TeamArgs {
@@ -276,36 +278,38 @@ __device__ __forceinline__ int gather_part(int n16) {
     return (n16 + NBC * U - 1) / (NBC * U) * U;
 }
 
-// One accumulator of a row pair of right-hand sides, added to R and I: the row's
-// real parts (lane t/4) and imaginary parts (lane t/4 + 8) times q's re hi, im hi,
-// re lo, im lo; with split operators the products of their lo parts with q's hi
-// parts 16 lanes further on.  The accumulators cover successive runs of input
-// chunks and are added here in rounded FP32: the tensor core's own additions do not
-// round to nearest, and the error of an apply grows with their chain (n = 31, one
-// front: 8.4e-6 with 2 accumulators, 6.5e-6 with 4).
-template <int RG>
-__device__ __forceinline__ void add_rows(uint32_t ta, bool split, float (&R)[4], float (&I)[4]) {
-    float rh[4], mh[4], rl[4], ml[4], lr[4] = {0.f, 0.f, 0.f, 0.f}, lm[4] = {0.f, 0.f, 0.f, 0.f};
-    __syncwarp();                                    // the TMEM loads are warp-collective
-    ptx::tmem_ld16x8(ta, rh);
-    ptx::tmem_ld16x8(ta + RG, mh);
-    ptx::tmem_ld16x8(ta + 2 * RG, rl);
-    ptx::tmem_ld16x8(ta + 3 * RG, ml);
-    if (split) {
-        ptx::tmem_ld16x8(ta + (16u << 16), lr);
-        ptx::tmem_ld16x8(ta + (16u << 16) + RG, lm);
-    }
-    ptx::tmem_wait_ld();
-    ptx::reg_tie4(rh);
-    ptx::reg_tie4(mh);
-    ptx::reg_tie4(rl);
-    ptx::reg_tie4(ml);
-    ptx::reg_tie4(lr);
-    ptx::reg_tie4(lm);
+// An accumulator's rows of a thread, for one pair of right-hand sides: of the row in
+// lane t/4 its real parts, 8 lanes on its imaginary parts, times q's re hi, im hi, re
+// lo, im lo (8 columns each); with split operators the products of their lo parts with
+// q's hi parts 16 lanes further on.
+struct AccRows {
+    float h[4][4], l[2][4];
+};
+__device__ __forceinline__ void load_rows(uint32_t ta, bool split, AccRows& v) {
+    ptx::tmem_ld16x32(ta, v.h);
+    if (split) ptx::tmem_ld16x16(ta + (16u << 16), v.l);
+}
+// Adds them to R and I after the wait.  The accumulators cover successive runs of the
+// input (Shape) and are added here in rounded FP32: the tensor core's own additions do
+// not round to nearest, and the error of an apply grows with their chain.
+__device__ __forceinline__ void add_rows(AccRows& v, bool split, float (&R)[4], float (&I)[4]) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        R[q] += rh[q] + (rl[q] + lr[q]);
-        I[q] += mh[q] + (ml[q] + lm[q]);
+    for (int q = 0; q < 4; ++q) ptx::reg_tie4(v.h[q]);
+    if (split) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) ptx::reg_tie4(v.l[q]);
+#pragma unroll
+        for (int q = 0; q < 4; q += 2) {
+            ptx::add2(v.h[2] + q, v.l[0] + q);
+            ptx::add2(v.h[3] + q, v.l[1] + q);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q += 2) {
+        ptx::add2(v.h[0] + q, v.h[2] + q);
+        ptx::add2(v.h[1] + q, v.h[3] + q);
+        ptx::add2(R + q, v.h[0] + q);
+        ptx::add2(I + q, v.h[1] + q);
     }
 }
 
@@ -332,24 +336,28 @@ __device__ __forceinline__ unsigned half_pow2(int d) {
 // takes 38 cycles where a 64-row product for hi and one for lo take 65; without, 64
 // rows.  One elected lane of the converged warp issues them; a full chunk is
 // straight-line code: a condition around each, even a uniform one, made a product
-// take 70 to 85 cycles to issue instead of 33.
+// take 70 to 85 cycles to issue instead of 33.  rsh: an accumulator takes 1 << rsh
+// products, or (2) whole chunks; add: the chunk goes on with its accumulator.
 template <int RG, int NSUB>
 __device__ __forceinline__ void chunk_products(uint32_t d, uint64_t ad, uint32_t sub, uint64_t bd, uint32_t idesc, uint32_t add,
-                                               int kc) {
-    constexpr int BSTEP = 2 * 64 * RG / 16, ASTEP = 256 / 16, SUBC = NACC * 4 * RG;
+                                               int rsh, int kc) {
+    constexpr int BSTEP = 2 * 64 * RG / 16, ASTEP = 256 / 16, SUBC = acc_slots(RG, 64 * NSUB) * 4 * RG;
+    const uint32_t mask = (1u << rsh) - 1u;
     if (kc == TKC) {
 #pragma unroll
         for (int ks = 0; ks < TKC / 16; ++ks)
 #pragma unroll
             for (int u = 0; u < NSUB; ++u)
-                ptx::umma_f16_warp(d + u * SUBC, ad + ks * ASTEP + u * sub, bd + ks * BSTEP, idesc, ks == 0 ? add : 1u);
+                ptx::umma_f16_warp(d + ((uint32_t)ks >> rsh) * (4 * RG) + u * SUBC, ad + ks * ASTEP + u * sub, bd + ks * BSTEP, idesc,
+                                   ks == 0 ? add : ks & mask);
         return;
     }
 #pragma unroll 1
     for (int ks = 0; 16 * ks < kc; ++ks) {
 #pragma unroll
-        for (int u = 0; u < NSUB; ++u) ptx::umma_f16_warp(d + u * SUBC, ad + ks * ASTEP + u * sub, bd + ks * BSTEP, idesc, add);
-        add = 1u;
+        for (int u = 0; u < NSUB; ++u)
+            ptx::umma_f16_warp(d + ((uint32_t)ks >> rsh) * (4 * RG) + u * SUBC, ad + ks * ASTEP + u * sub, bd + ks * BSTEP, idesc,
+                               ks == 0 ? add : ks & mask);
     }
 }
 
@@ -359,9 +367,20 @@ __device__ __forceinline__ void chunk_products(uint32_t d, uint64_t ad, uint32_t
 // that the step loops carry no index divisions (inlined in every role they made
 // the code larger than the instruction caches: 258 kB and 5 to 8 cycles per
 // instruction).
+//
+// An accumulator takes a run of products: a quarter of the input's, an eighth beyond 32
+// products, rounded down to 1, 2 or a multiple of 4 so that runs and chunks end together.  The products signal a few accumulators at a
+// time, a unit: those of a chunk, or two, or one where there are at most four.  Before the
+// teams every input went into eight partial sums; error of a split FP16 apply against 64
+// bits then, with four accumulators of whole chunks, and now: n = 33, two fronts, b_aux 1 (6
+// products, so two accumulators) 6.4e-6, 8.0e-6, 4.6e-6; n = 50, one front, b_aux 3 (16)
+// 8.9e-6, 8.5e-6, 8.5e-6; the same with d = 2 (39) 8.1e-6, 6.7e-6, 4.3e-6.  Reading an accumulator costs a warp 150 cycles or more: runs of
+// an eighth for all give n = 50 6.0e-6 in 64.8 ms instead of 60.2, n = 63 with one right-hand
+// side 43.2 ms instead of 40.6.
 enum { KIND_START = 0, KIND_RING = 1, KIND_CENTRE = 2, KIND_END = 3 };
 struct Shape {
-    int K, KP, nch, nacc;         // input entries, padded; chunks; accumulators
+    int K, KP;                    // input entries, padded to a multiple of 16
+    int rsh, cpa, nu, w, wl;      // chunk_products' rsh, chunks of an accumulator, units of a tile, accumulators of each and of the last
     int a0, c0, a1, c1;           // this rank's row groups [a, a + c) of the two out rects
     int ng0, ng, nt, kg0;         // row groups of rect 0 and of the operator, tiles, first own input group
     int kg1, nl, nz, z0;          // end of the own input groups; the in rect's lines, z rows and first row
@@ -383,8 +402,6 @@ __device__ __noinline__ void make_shapes(Shape* out, const AxisWin* win, int N, 
         Shape s;
         s.K = g.K;
         s.KP = tm_kp(g.K);
-        s.nch = tm_ceil(s.KP, TKC);
-        s.nacc = min(NACC, s.nch);
         int hi;
         tm_part(g.n0, g.out0.nl, g.f0, rank, C, &s.a0, &hi);
         s.c0 = hi - s.a0;
@@ -396,6 +413,13 @@ __device__ __noinline__ void make_shapes(Shape* out, const AxisWin* win, int N, 
         s.ng0 = tm_ceil(g.n0, 8);
         s.ng = s.ng0 + tm_ceil(g.n1, 8);
         s.nt = tm_ceil(s.c0 + s.c1, GT);
+        const int n16 = s.KP / 16, nch = tm_ceil(s.KP, TKC), run = tm_ceil(n16, n16 <= 32 ? 4 : 8);
+        s.rsh = run >= 4 ? 2 : (run > 1 ? 1 : 0);
+        s.cpa = max(1, run / 4);
+        const int na = run >= 4 ? tm_ceil(nch, s.cpa) : tm_ceil(n16, 1 << s.rsh);
+        s.w = run == 1 ? 4 : (run >= 4 && na <= 4 ? 1 : 2);
+        s.nu = s.nt > 0 ? tm_ceil(na, s.w) : 1;
+        s.wl = na - (tm_ceil(na, s.w) - 1) * s.w;
         tm_part(g.K, g.in.nl, g.fin, rank, C, &s.kg0, &s.kg1);
         s.nl = g.in.nl;
         s.nz = g.in.nz;
@@ -414,8 +438,9 @@ struct Sm {
     uint64_t bgo;                // a gather pass may be multiplied
     uint64_t eready;             // its scale exponents are in shared memory
     uint64_t mdone;              // its products are complete
-    uint64_t sacc[NACC - 1];     // an accumulator's products are complete (one tile; otherwise with sdone)
-    uint64_t sdone;              // a tile batch's products are complete
+    uint64_t sacc[8];            // a unit's products are complete, by its place in TMEM
+    uint64_t afree[8];           // its accumulators have been read (CW arrivals), where another unit of the tile follows
+    uint64_t sdone;              // a tile's products are complete (stands for its last unit)
     uint64_t tfree;              // its accumulators have been read (CW arrivals)
     uint64_t cbar;               // barrier of the update warps (CW arrivals)
     uint64_t xbar;               // teardown
@@ -441,7 +466,7 @@ struct Sm {
 
 // An update warp's place in the barriers' phases.
 struct Upd {
-    uint32_t sph, cph, xph;      // sph: a parity bit per accumulator, the last for sdone
+    uint32_t sph, cph, xph;      // sph: a parity bit per place of a unit, bit 8 for sdone
     unsigned arrivals, tag;      // tag: number of the solve, from 1
 };
 
@@ -454,11 +479,9 @@ __device__ __forceinline__ int warp_of(int gi, int pcb) {
     return MT == 64 ? gi & 3 : gi & 7;
 }
 // Where a lane's part of a row lies in its group of 8 entries, for right-hand sides
-// 8 pcb ..: part lane mod 4 (re hi, im hi, re lo, im lo) of row lane / 4.
-template <int RG>
-__device__ __forceinline__ int part_offset(int pcb, int lane) {
-    return ((lane & 3) * (RG / 8) + pcb) * 128 + (lane >> 2) * 16;
-}
+// 8 pcb ..: part lane mod 4 (re hi, im hi, re lo, im lo) of row lane / 4.  A block of
+// right-hand sides has its four parts side by side, 32 accumulator columns for one load.
+__device__ __forceinline__ int part_offset(int pcb, int lane) { return (pcb * 4 + (lane & 3)) * 128 + (lane >> 2) * 16; }
 __device__ __forceinline__ void fail(const TeamArgs& A, Sm& S) {
     if (!S.abort) atomicOr(A.err, 2);
     S.abort = 1;
@@ -502,6 +525,44 @@ __device__ __forceinline__ void release_header(u64* hd, unsigned w, unsigned tag
 __device__ __forceinline__ void store_header(u64* hd, unsigned w, unsigned tag) {
     const int lane = threadIdx.x & 31;
     if (lane < 4) ptx::st_relaxed_gpu_u64(hd + lane, (u64)tag << 32 | w);
+}
+
+// A warp's rows of a tile: the sum of its accumulators, read as their units complete
+// while the next ones are multiplied.  fv: whether the warp has rows (the second group's
+// sums are of no use where it does not exist).
+template <int RG, int MT, int NRS>
+__device__ __forceinline__ bool read_tile(Sm& T, Upd& u, const Shape& S, uint32_t tlane, bool split, bool fv,
+                                          float (&R)[NRS][4], float (&I)[NRS][4]) {
+    constexpr int SLOTS = acc_slots(RG, MT), SUBC = SLOTS * 4 * RG;
+    const int nu = S.nu, w = S.w, NU = SLOTS >> (w >> 1);
+    int s = 0;
+#pragma unroll 1
+    for (int a = 0; a < nu; ++a) {
+        const bool last = a == nu - 1;
+        const int b = last ? 8 : s;
+        if (!wait_phase(last ? &T.sdone : &T.sacc[s], u.sph >> b & 1u, T.limit, &T.abort)) return false;
+        u.sph ^= 1u << b;
+        ptx::tc_fence_after();
+        const int n = last ? S.wl : w;
+        __syncwarp();                                // the TMEM loads are warp-collective
+        if (fv)
+#pragma unroll 1
+            for (int v = 0; v < n; ++v)
+#pragma unroll
+                for (int j = 0; j < NRS; ++j) {
+                    AccRows t;
+                    load_rows(tlane + (s * w + v) * 4 * RG + j * SUBC, split, t);
+                    ptx::tmem_wait_ld();
+                    add_rows(t, split, R[j], I[j]);
+                }
+        if (a + NU < nu) {
+            ptx::tc_fence_before();
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(&T.afree[s]);
+        }
+        if (++s == NU) s = 0;
+    }
+    return true;
 }
 
 // Boundary of slab visits jo-1 and jo (Algorithm 6).
@@ -617,17 +678,17 @@ __device__ __noinline__ void boundary_phase(const TeamArgs& A, Sm* T, int jo) {
         gm[((jo + 1) & 1) * N * RG + q] = 0u;
 }
 
-// Updates of a tile batch of any shape: couplings go through FP32 buffers.
+// Updates of a tile of any shape: couplings go through FP32 buffers.
 template <int RG, int MT>
-__device__ __noinline__ void general_rows(const TeamArgs& A, Sm* T, int M, int i, int tb, long long soff,
+__device__ __noinline__ bool general_rows(const TeamArgs& A, Sm* T, Upd* pu, int M, int i, int tl, long long soff,
               uint32_t tmem, int ec0, int ec1) {
-    constexpr int GT = MT / 16, NRS = RG == 16 && MT == 128 ? 2 : 1, SUBC = NACC * 4 * RG, TCOLS = MT / 64 * SUBC, TBATCH = 512 / TCOLS;
+    constexpr int GT = MT / 16, NRS = RG == 16 && MT == 128 ? 2 : 1, SUBC = acc_slots(RG, MT) * 4 * RG;
     const int N = T->N, B = T->B, cen = T->cen, two = T->two, U = T->U, team = T->team, VL = T->VL, GL = T->GL;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q4 = warp & 3, hh = warp >> 2, ii = lane >> 2, c = lane & 3;
     const int cb = RG == 16 ? hh : 0, rhs0 = 8 * cb + 2 * c;
     const int gi0 = RG == 8 && MT == 128 ? warp : q4;
     const bool idle = RG == 8 && MT == 64 && hh == 1;
-    const uint32_t tlane = tmem + ((uint32_t)(32 * q4) << 16) + 8 * cb + (gi0 >> 2) * SUBC;
+    const uint32_t tlane = tmem + ((uint32_t)(32 * q4) << 16) + 32 * cb + (gi0 >> 2) * SUBC;
     const int nsol = tm_solves(B, cen, team);
     const TeamSolve t = tm_solve(i, B, cen, team);
     const AxisWin wz = T->win[M], wy = T->win[t.Mp];
@@ -644,20 +705,24 @@ __device__ __noinline__ void general_rows(const TeamArgs& A, Sm* T, int M, int i
     const SolveGeo g = tm_geo(wz, wy, N, t.Mp, t.bwd, B, two);
     const int lc = (t.bwd ? t.role == ROLE_L : t.role != ROLE_L) ? y0 : y1 - 1;   // the line that feeds the next
     float2* qb = Qf + (into_centre ? team : (centre && two ? 0 : 2 + team)) * VL;
-#pragma unroll 1
-    for (int tl = tb; tl < min(S.nt, tb + TBATCH); ++tl)
-#pragma unroll 1
-        for (int j = 0; j < NRS; ++j) {
-            const int pos = tl * GT + gi0 + 4 * j;
-            if (idle || pos >= S.c0 + S.c1) continue;      // the same in the whole warp
+    const int p0 = tl * GT + gi0, np = S.c0 + S.c1;
+    float R[NRS][4] = {}, I[NRS][4] = {};
+    Upd u = *pu;
+    const bool ok = read_tile<RG, MT, NRS>(*T, u, S, tlane, A.halves == 2, !idle && p0 < np, R, I);
+    *pu = u;
+    if (!ok) return false;
+    ptx::tc_fence_before();
+    __syncwarp();
+    if (lane == 0) ptx::mbar_arrive(&T->tfree);
+#pragma unroll
+    for (int j = 0; j < NRS; ++j) {
+        const int pos = p0 + 4 * j;
+        if (!idle && pos < np) {                           // the same in the whole warp
             const int rect = pos >= S.c0, gid = rect ? S.a1 + pos - S.c0 : S.a0 + pos;
             const int r = 8 * gid + ii;
             const int nl = rect ? g.out1.nl : g.out0.nl, nz = rect ? g.out1.nz : g.out0.nz;
             const float* sc = A.scale + soff + (long long)((rect ? S.ng0 : 0) + gid) * 16 + ii;
-            float R[4] = {0.f, 0.f, 0.f, 0.f}, I[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int a = 0; a < S.nacc; ++a)
-                add_rows<RG>(tlane + (uint32_t)(j * SUBC + (tl - tb) * TCOLS + a * 4 * RG), A.halves == 2, R, I);
-            float4 X = scale_rows(R, I, (__float_as_int(__ldg(sc)) >> 23) - 127, (__float_as_int(__ldg(sc + 8)) >> 23) - 127,
+            float4 X = scale_rows(R[j], I[j], (__float_as_int(__ldg(sc)) >> 23) - 127, (__float_as_int(__ldg(sc + 8)) >> 23) - 127,
                                   ec0, ec1);
             if (r < (rect ? g.n1 : g.n0)) {
                 const int l = r % nl, tt = r / nl, x = tt / nz;
@@ -674,6 +739,8 @@ __device__ __noinline__ void general_rows(const TeamArgs& A, Sm* T, int M, int i
             }
             __syncwarp();
         }
+    }
+    return true;
 }
 
 // Publishes the rank's entries of an input of the given kind for team T->team + up,
@@ -721,7 +788,7 @@ __device__ __noinline__ void publish_input(const TeamArgs& A, Sm* T, int jo, int
             if (l == l1) v = add4(v, __ldcg(reinterpret_cast<const float4*>(b1 + eo)));
             if (l == l2) v = add4(v, __ldcg(reinterpret_cast<const float4*>(b2 + eo)));
         }
-        const unsigned w = store_parts(xs + (size_t)kg * KGB + part_offset<RG>(pcb, lane), v, e0, e1);
+        const unsigned w = store_parts(xs + (size_t)kg * KGB + part_offset(pcb, lane), v, e0, e1);
 #pragma unroll
         for (int q = 0; q < PB; ++q)
             if (q == held) {
@@ -743,14 +810,6 @@ __device__ __noinline__ void publish_input(const TeamArgs& A, Sm* T, int jo, int
         for (int q = 0; q < PB; ++q)
             if (q < held) store_header(hp[q], hw[q], tag);
     }
-}
-
-// Waits until accumulator a of nacc has all its products.
-__device__ __forceinline__ bool wait_acc(Sm& T, Upd& u, int a, int nacc, long long limit) {
-    const int b = a == nacc - 1 ? NACC - 1 : a;
-    const bool r = wait_phase(b == NACC - 1 ? &T.sdone : &T.sacc[b], u.sph >> b & 1u, limit, &T.abort);
-    u.sph ^= 1u << b;
-    return r;
 }
 
 // Barrier of the update warps.
@@ -856,12 +915,13 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
     const int rhs0 = 8 * cb + 2 * c;                      // this thread's right-hand sides rhs0, rhs0 + 1
     const int gi0 = RG == 8 && MT == 128 ? warp : q4;     // its first row group of a tile (the second: 4 on)
     const bool idle = RG == 8 && MT == 64 && hh == 1;     // no accumulator columns for this warp
-    constexpr int SUBC = NACC * 4 * RG;
-    const uint32_t tlane = T.tslot + ((uint32_t)(32 * q4) << 16) + 8 * cb + (gi0 >> 2) * SUBC;
+    constexpr int SUBC = acc_slots(RG, MT) * 4 * RG;
+    const uint32_t tlane = T.tslot + ((uint32_t)(32 * q4) << 16) + 32 * cb + (gi0 >> 2) * SUBC;
     const bool split = A.halves == 2;
     const int B = T.B, cen = T.cen, team = T.team, nsol = T.nsol;
     const AxisWin wz = T.win[pass_pos(jo, B, cen).M];
-    const int Lz = wz.L, za = wz.ia, dz = wz.ib - wz.ia, E = T.N * Lz, KP = tm_kp(E);
+    const int Lz = wz.L, za = wz.ia, dz = wz.ib - wz.ia, E = T.N * Lz;
+    const Shape& S = T.shape[8 + KIND_RING];
     int cg0, cg1;                                         // this rank's groups of 8 columns
     tm_part(E, 1, 1, T.rank, T.C, &cg0, &cg1);
     cg0 += gi0;                                           // this warp's (first) group
@@ -885,10 +945,9 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
     const float2* gl = T.Gv + (y + dy) * T.GL;            // the right-hand side on the next line
     float2* zl = T.Zv + y * T.GL;
     const int VL = T.VL * dy, GL = T.GL * dy;
-    unsigned char* X = T.X + (size_t)cg0 * KGB + part_offset<RG>(cb, lane);    // this thread's parts in slot 0
+    unsigned char* X = T.X + (size_t)cg0 * KGB + part_offset(cb, lane);    // this thread's parts in slot 0
     u64* H = T.H + (cg0 * NB + cb) * 4;
     const float* scale = A.scale + cg0 * 16 + ii;
-    const int nacc = min(NACC, tm_ceil(KP, TKC));
     int ri = slot_of_solve(i, nsol, cen, team);           // ring slot of solve i
     Upd u = *up;
     bool ok = true;
@@ -915,17 +974,8 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
         u.xph ^= 1u;
         if (!ok) break;
         const int2 ec = *reinterpret_cast<const int2*>(&T.ecol[rhs0]), ep = *reinterpret_cast<const int2*>(&T.epred[rhs0]);
-        // accumulators are read as they complete, while the next one is multiplied
         float R[NRS][4] = {}, I[NRS][4] = {};
-#pragma unroll 1
-        for (int a = 0; a < nacc && ok; ++a) {
-            if (!(ok = wait_acc(T, u, a, nacc, T.limit))) break;
-            ptx::tc_fence_after();
-#pragma unroll
-            for (int j = 0; j < NRS; ++j)
-                if (j ? fv1 : fv) add_rows<RG>(tlane + j * SUBC + a * 4 * RG, split, R[j], I[j]);
-        }
-        if (!ok) break;
+        if (!(ok = read_tile<RG, MT, NRS>(T, u, S, tlane, split, fv, R, I))) break;
         float4 W[NRS];
 #pragma unroll
         for (int j = 0; j < NRS; ++j)
@@ -981,7 +1031,6 @@ __device__ __forceinline__ int lines_end(Sm& T, int jo, int i) {
 template <int RG, int MT>
 __device__ __noinline__ bool run_general(const TeamArgs& A, Sm* Tp, Upd* up, int jo, int i) {
     Sm& T = *Tp;
-    constexpr int TBATCH = 512 / (MT / 64 * NACC * 4 * RG);
     const int lane = threadIdx.x & 31, c = lane & 3, rhs0 = 8 * (RG == 16 ? (int)(threadIdx.x >> 7) : 0) + 2 * c;
     const int B = T.B, cen = T.cen, team = T.team, nsol = T.nsol, U = T.U;
     const bool two = T.two;
@@ -996,20 +1045,14 @@ __device__ __noinline__ bool run_general(const TeamArgs& A, Sm* Tp, Upd* up, int
     Upd u = *up;
     ++u.tag;
     bool ok = true;
+    ok = wait_phase(&T.eready, u.xph, limit, &T.abort);
+    u.xph ^= 1u;
+    *up = u;
+    const int ec0 = T.ecol[rhs0], ec1 = T.ecol[rhs0 + 1];
 #pragma unroll 1
-    for (int tb = 0; (tb < S.nt || tb == 0) && ok; tb += TBATCH) {
-        if (tb == 0) {
-            ok = wait_phase(&T.eready, u.xph, limit, &T.abort);
-            u.xph ^= 1u;
-        }
-        for (int a = 0; a < S.nacc && ok; ++a) ok = wait_acc(T, u, a, S.nacc, limit);
-        if (!ok) break;
-        ptx::tc_fence_after();
-        general_rows<RG, MT>(A, Tp, M, i, tb, T.soff[op_slot(t.Mp, t.bwd, B)], T.tslot, T.ecol[rhs0], T.ecol[rhs0 + 1]);
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(&T.tfree);
-    }
+    for (int tl = 0; (tl < S.nt || tl == 0) && ok; ++tl)
+        ok = general_rows<RG, MT>(A, Tp, up, M, i, tl, T.soff[op_slot(t.Mp, t.bwd, B)], T.tslot, ec0, ec1);
+    u = *up;
     if (ok && more && !into_centre) {
         ok = cta_sync(T, u, limit);
         if (ok) {
@@ -1040,8 +1083,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
     constexpr int GT = MT / 16;              // row groups of a tile
     constexpr int ACOLS = 4 * RG;            // columns of an accumulator: G times q's re hi, im hi, re lo, im lo
     constexpr int NSUB = MT / 64;            // products of 4 row groups per tile and 16 input entries
-    constexpr int TCOLS = NSUB * NACC * ACOLS;   // accumulator columns of a tile
-    constexpr int TBATCH = 512 / TCOLS;      // tiles with accumulators at a time
+    constexpr int SLOTS = acc_slots(RG, MT); // accumulators of each
     const int B = A.g.B, N = A.g.N, cen = A.g.cen;
     const int two = A.T == 2;
     unsigned char* ring = smem;
@@ -1075,7 +1117,10 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
         ptx::mbar_init(eready, 1);
         ptx::mbar_init(mdone, 1);
         ptx::mbar_init(sdone, 1);
-        for (int q = 0; q < NACC - 1; ++q) ptx::mbar_init(&S_.sacc[q], 1);
+        for (int q = 0; q < 8; ++q) {
+            ptx::mbar_init(&S_.sacc[q], 1);
+            ptx::mbar_init(&S_.afree[q], CW);
+        }
         ptx::mbar_init(tfree, CW);
         ptx::mbar_init(&S_.cbar, CW);
         ptx::mbar_init(&S_.xbar, 1);
@@ -1131,34 +1176,29 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                 const int c0 = S.c0, cs = c0 + S.c1, nt = S.nt, KP = S.KP, ng = S.ng;
                 const unsigned char* base = A.G + s_off[op_slot(t.Mp, t.bwd, B)];
 #pragma unroll 1
-                for (int tb = 0; tb < nt && ok; tb += TBATCH)
+                for (int tl = 0; tl < nt && ok; ++tl) {
+                    // the tile's groups: at most two runs of stored groups (lane & 1: this lane's)
+                    const int g0 = tl * GT, g1 = min(cs, g0 + GT);
+                    const int m0 = max(0, min(g1, c0) - g0);
+                    const int run = lane & 1;
+                    const int cnt = run ? g1 - g0 - m0 : m0;
+                    const int gr = run ? S.ng0 + S.a1 + max(0, g0 - c0) : S.a0 + g0;
 #pragma unroll 1
-                    for (int k0 = 0; k0 < KP && ok; k0 += A.KB)
-#pragma unroll 1
-                        for (int tl = tb; tl < min(nt, tb + TBATCH) && ok; ++tl) {
-                            // the tile's groups: at most two runs of stored groups (lane & 1: this lane's)
-                            const int g0 = tl * GT, g1 = min(cs, g0 + GT);
-                            const int m0 = max(0, min(g1, c0) - g0);
-                            const int run = lane & 1;
-                            const int cnt = run ? g1 - g0 - m0 : m0;
-                            const int gr = run ? S.ng0 + S.a1 + max(0, g0 - c0) : S.a0 + g0;
-                            const int kend = min(KP, k0 + A.KB);
-#pragma unroll 1
-                            for (int kc0 = k0; kc0 < kend; kc0 += TKC) {
-                                ok = wait_phase(&empty[stage], eph, limit, s_abort);
-                                if (!ok) break;
-                                const int kc = min(TKC, KP - kc0), per = 32 * kc * A.halves;      // bytes of a group
-                                if (lane == 0)
-                                    ptx::mbar_expect_tx(&full[stage], (uint32_t)((g1 - g0) * per));
-                                __syncwarp();
-                                if (lane < 2 && cnt > 0)
-                                    ptx::bulk_g2s(ring + stage * A.stage_bytes + (run ? m0 : 0) * per,
-                                                  base + ((size_t)kc0 * ng + (size_t)kc * gr) * A.halves * 32,
-                                                  (uint32_t)(cnt * per), &full[stage]);
-                                ++issued;
-                                if (++stage == A.stages) { stage = 0; eph ^= 1u; }
-                            }
-                        }
+                    for (int kc0 = 0; kc0 < KP; kc0 += TKC) {
+                        ok = wait_phase(&empty[stage], eph, limit, s_abort);
+                        if (!ok) break;
+                        const int kc = min(TKC, KP - kc0), per = 32 * kc * A.halves;      // bytes of a group
+                        if (lane == 0)
+                            ptx::mbar_expect_tx(&full[stage], (uint32_t)((g1 - g0) * per));
+                        __syncwarp();
+                        if (lane < 2 && cnt > 0)
+                            ptx::bulk_g2s(ring + stage * A.stage_bytes + (run ? m0 : 0) * per,
+                                          base + ((size_t)kc0 * ng + (size_t)kc * gr) * A.halves * 32,
+                                          (uint32_t)(cnt * per), &full[stage]);
+                        ++issued;
+                        if (++stage == A.stages) { stage = 0; eph ^= 1u; }
+                    }
+                }
             }
         }
         if (!ok) fail(A, S_);
@@ -1180,7 +1220,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
         const uint64_t bdesc0 = ptx::umma_desc(ptx::smem_u32(Bbuf), KGB, 128u);
         const uint32_t a_s = ptx::smem_u32(ring);
         int stage = 0, seen = 0;                                  // seen: chunks ahead known to have landed
-        uint32_t fph = 0, gph = 0, tph = 1, bph = 0;              // bph: a parity bit per part
+        uint32_t fph = 0, gph = 0, tph = 1, bph = 0, aph = 0;     // bph, aph: a parity bit per part and per place of a unit
         bool ok = true;
         for (int jo = 0; jo < nvis && ok; ++jo) {
 #pragma unroll 1
@@ -1197,67 +1237,69 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                 if (!(ok = wait_phase(bgo, gph, limit, s_abort))) break;    // of the solve's first gather
                 const Shape& S = shapes[kind_of(i, nsol, cen, team)];
                 const int KP = __shfl_sync(0xffffffffu, S.KP, 0), nt = __shfl_sync(0xffffffffu, S.nt, 0);
-                const int nch = __shfl_sync(0xffffffffu, S.nch, 0), nacc = __shfl_sync(0xffffffffu, S.nacc, 0);
+                const int nu = __shfl_sync(0xffffffffu, S.nu, 0), cpa = __shfl_sync(0xffffffffu, S.cpa, 0);
+                const int w = __shfl_sync(0xffffffffu, S.w, 0), NU = SLOTS >> (w >> 1);
+                const int rsh = __shfl_sync(0xffffffffu, S.rsh, 0), per = rsh == 2 ? 1 : w;   // per: accumulators of a chunk or run
+                const bool passes = KP > A.KB;                    // every tile gathers the input anew, in passes
 #pragma unroll 1
-                for (int tb = 0; (tb < nt || tb == 0) && ok; tb += TBATCH) {
-                    if (tb > 0) {                                 // so has the batch before
+                for (int tl = 0; (tl < nt || tl == 0) && ok; ++tl) {
+                    if (tl > 0) {                                 // the tile before has been read out too
                         if (!(ok = wait_phase(tfree, tph, limit, s_abort))) break;
                         tph ^= 1u;
                     }
+                    int un = 0, us = 0, va = 0, ca = 0;           // unit, its place, accumulators done, chunks of the next
 #pragma unroll 1
                     for (int k0 = 0; k0 < KP && ok; k0 += A.KB) {
                         const int ke = min(KP, k0 + A.KB), part = 16 * gather_part((ke - k0) >> 4);
-                        if (tb + k0 > 0 && !(ok = wait_phase(bgo, gph, limit, s_abort))) break;
-                        gph ^= 1u;
-#pragma unroll 1
-                        for (int tl = tb; (tl < min(nt, tb + TBATCH) || tl == tb) && ok; ++tl) {
-                            // an accumulator takes a run of the chunks: chunk ch goes to accumulator ch nacc / nch
-                            int ac = k0 / TKC * nacc, acc = 0;
-                            while (ac >= nch) { ac -= nch; ++acc; }
-                            int fresh = ac < nacc;                // the chunk is its accumulator's first
-                            uint64_t bd = bdesc0;
-#pragma unroll 1
-                            for (int kc0 = k0, pj = 0; kc0 < ke; ++pj) {
-                                if (tl == tb) {                   // the pass's first tile sees every part
-                                    if (!(ok = wait_phase(&bfull[pj], bph >> pj & 1u, limit, s_abort))) break;
-                                    bph ^= 1u << pj;
-                                }
-                                const int kpe = min(ke, kc0 + part);
-                                if (tl >= nt) kc0 = kpe;          // a rank without rows only sees them
-                                ptx::tc_fence_after();
-#pragma unroll 1
-                                for (; kc0 < kpe; kc0 += TKC) {
-                                    const int kc = min(TKC, KP - kc0);
-                                    if (--seen < 0) {
-                                        seen = 0;
-                                        if (!(ok = wait_phase(&full[stage], fph, limit, s_abort))) break;
-                                        ptx::tc_fence_after();
-                                    }
-                                    const uint32_t d = tmem + (uint32_t)((tl - tb) * TCOLS + acc * ACOLS);
-                                    const uint32_t ahi = a_s + (uint32_t)(stage * A.stage_bytes), sbo = (uint32_t)(kc * 16);
-                                    chunk_products<RG, NSUB>(d, ptx::umma_desc(ahi, 128u, sbo), 8 * A.halves * sbo / 16, bd, idesc,
-                                                             !fresh, kc);
-                                    bd += TKC / 16 * 2 * KGB / 16;
-                                    ptx::umma_commit_warp(&empty[stage]);
-                                    if (++stage == A.stages) { stage = 0; fph ^= 1u; }
-                                    ac += nacc;
-                                    fresh = ac >= nch;
-                                    if (fresh) {
-                                        if (nt == 1 && acc < nacc - 1) ptx::umma_commit_warp(&S_.sacc[acc]);
-                                        ac -= nch;
-                                        ++acc;
-                                    }
-                                }
-                                if (!ok) break;
-                            }
+                        const bool gathered = tl == 0 || passes;  // a gather of its own: wait for its parts
+                        if (gathered) {
+                            if (tl + k0 > 0 && !(ok = wait_phase(bgo, gph, limit, s_abort))) break;
+                            gph ^= 1u;
                         }
-                        if (ok) ptx::umma_commit_warp(mdone);
+                        uint64_t bd = bdesc0;
+#pragma unroll 1
+                        for (int kc0 = k0, pj = 0; kc0 < ke; ++pj) {
+                            if (gathered) {
+                                if (!(ok = wait_phase(&bfull[pj], bph >> pj & 1u, limit, s_abort))) break;
+                                bph ^= 1u << pj;
+                            }
+                            const int kpe = min(ke, kc0 + part);
+                            if (nt == 0) kc0 = kpe;               // a rank without rows only sees them
+                            ptx::tc_fence_after();
+#pragma unroll 1
+                            for (; kc0 < kpe; kc0 += TKC) {
+                                const int kc = min(TKC, KP - kc0);
+                                if (--seen < 0) {
+                                    seen = 0;
+                                    if (!(ok = wait_phase(&full[stage], fph, limit, s_abort))) break;
+                                    ptx::tc_fence_after();
+                                }
+                                if (un >= NU && va + ca == 0) {   // the unit there before has been read
+                                    if (!(ok = wait_phase(&S_.afree[us], aph >> us & 1u, limit, s_abort))) break;
+                                    aph ^= 1u << us;
+                                    ptx::tc_fence_after();
+                                }
+                                const uint32_t d = tmem + (uint32_t)((us * w + va) * ACOLS);
+                                const uint32_t ahi = a_s + (uint32_t)(stage * A.stage_bytes), sbo = (uint32_t)(kc * 16);
+                                const uint64_t ad = ptx::umma_desc(ahi, 128u, sbo);
+                                chunk_products<RG, NSUB>(d, ad, 8 * A.halves * sbo / 16, bd, idesc, ca > 0, rsh, kc);
+                                bd += TKC / 16 * 2 * KGB / 16;
+                                ptx::umma_commit_warp(&empty[stage]);
+                                if (++stage == A.stages) { stage = 0; fph ^= 1u; }
+                                if (++ca == cpa) {
+                                    ca = 0;
+                                    if ((va += per) == w) {
+                                        va = 0;
+                                        if (++un < nu) ptx::umma_commit_warp(&S_.sacc[us]);
+                                        if (++us == NU) us = 0;
+                                    }
+                                }
+                            }
+                            if (!ok) break;
+                        }
+                        if (ok && (passes || tl + 1 >= nt)) ptx::umma_commit_warp(mdone);
                     }
-                    if (ok) {
-                        if (nt != 1)
-                            for (int q = 0; q < nacc - 1; ++q) ptx::umma_commit_warp(&S_.sacc[q]);
-                        ptx::umma_commit_warp(sdone);
-                    }
+                    if (ok) ptx::umma_commit_warp(sdone);
                 }
             }
         }
@@ -1361,12 +1403,13 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                 const bool none = lane >= nv;                         // fewer header words than lanes
                 const bool even = __all_sync(0xffffffffu, none || (((mx0 ^ mn0) | (mx1 ^ mn1) | (mx0 ^ x0) | (mx1 ^ x1)) &
                                                                     0xff00ff00u) == 0u);
+                // one gather for all tiles, or every tile's passes
 #pragma unroll 1
-                for (int tb = 0; (tb < nt || tb == 0) && ok; tb += TBATCH)
+                for (int tl = 0; (tl == 0 || (tl < nt && KP > A.KB)) && ok; ++tl)
 #pragma unroll 1
                     for (int k0 = 0; k0 < KP && ok; k0 += A.KB) {
                         // the pass before has been multiplied
-                        const bool first = tb == 0 && k0 == 0;
+                        const bool first = tl == 0 && k0 == 0;
                         if (!first) {
                             if (!(ok = wait_phase(mdone, mph, limit, s_abort))) break;
                             mph ^= 1u;
@@ -1421,7 +1464,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                             if (!ok) break;
 #pragma unroll 1
                             for (int v = lane; v < n16 * 2 * 4 * NB * 8; v += 32) {
-                                const int kg = v / (4 * NB * 8), b8 = (v >> 3) % NB;
+                                const int kg = v / (4 * NB * 8), b8 = (v >> 5) % NB;
                                 if (k0 / 8 + kg >= ng8) continue;
                                 const u64* hw = hw0 + ((size_t)(k0 / 8 + kg) * NB + b8) * 4;
                                 __half* p = reinterpret_cast<__half*>(Bbuf) + v * 8;
