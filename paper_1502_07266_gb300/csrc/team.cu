@@ -1314,7 +1314,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
         Shape* shapes = s_shape + 4;
         uint32_t mph = 0, lph = 0;           // lph: a bit per part, the phase its next copy completes
         bool ok = true, fresh = true;
-        unsigned tag = 0;
+        unsigned tag = 0, tiles = 0;         // tiles: of the solves before
         int ri = 0;
         // lane's header words: right-hand sides 8 cb + 4 cp .. + 3 of every group of 8 entries
         const int cp = lane & 1, cb = RG == 16 ? (lane >> 1) & 1 : 0;
@@ -1433,7 +1433,10 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                                 mn0 = __vminu4(mn0, __shfl_xor_sync(0xffffffffu, mn0, s));
                                 mn1 = __vminu4(mn1, __shfl_xor_sync(0xffffffffu, mn1, s));
                             }
-                            // scale exponents: of this input (the smallest used one), of the next
+                            // scale exponents: of this input (the smallest used one), of the next; every update
+                            // warp has read those of the solve before
+                            if (tiles > 0 && !(ok = wait_phase(tfree, (tiles - 1) & 1u, limit, s_abort))) break;
+                            tiles += max(nt, 1);
                             if (lane < 2 * NB) {
                                 float gn[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
