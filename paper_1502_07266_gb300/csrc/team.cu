@@ -45,7 +45,8 @@
 // streams the operator through a ring, one polls headers and gathers.  The loops
 // that run every solve are kept small and straight (the instruction cache holds 32
 // kB; code beyond it runs at a third of the rate and branchy code worse): solves of
-// one line in one tile run in run_lines, every other one in run_general.
+// one line in one tile run in run_lines, of 2 or 4 lines or of several tiles in
+// run_blocks, every other one in run_general.
 // All waits are bounded; on expiry the error word is set, copies and products in
 // flight are drained, TMEM is freed and the kernel returns.
 #include "helm_internal.h"
@@ -1014,17 +1015,132 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
     return ok;
 }
 
-// First solve after the run of run_lines that starts with solve i (i itself: none).
-template <int MT>
-__device__ __forceinline__ int lines_end(Sm& T, int jo, int i) {
+// The same for blocks of nl lines, 8 a multiple of nl, and for several tiles a rank.
+// A column's nl lines are neighbouring rows of one group, so the coupling gets from the
+// line that feeds the next block to the one that takes it by a shuffle, and a warp
+// publishes the groups whose rows it holds, each tile while the next is multiplied.
+// Against run_general (couplings through L2, a barrier of the CTA, index divisions
+// after the product) one apply: two lines, n = 50, one
+// front with 24 right-hand sides 31.0 -> 22.1 ms (the K split over clusters 25.3), n = 30, two
+// fronts with 9 6.7 -> 4.5 (5.4), n = 17 with two 1.90 -> 1.44 (1.71)
+template <int RG, int MT>
+__device__ __noinline__ bool run_blocks(const TeamArgs& A, Sm* Tp, Upd* up, int jo, int i, int end) {
+    Sm& T = *Tp;
+    constexpr int GT = MT / 16, NB = RG / 8, KGB = 64 * RG;
+    constexpr int NRS = RG == 16 && MT == 128 ? 2 : 1, SUBC = acc_slots(RG, MT) * 4 * RG;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q4 = warp & 3, hh = warp >> 2, ii = lane >> 2, c = lane & 3;
+    const int cb = RG == 16 ? hh : 0, rhs0 = 8 * cb + 2 * c;
+    const int gi0 = RG == 8 && MT == 128 ? warp : q4;
+    const bool idle = RG == 8 && MT == 64 && hh == 1;
+    const uint32_t tlane = T.tslot + ((uint32_t)(32 * q4) << 16) + 32 * cb + (gi0 >> 2) * SUBC;
+    const bool split = A.halves == 2;
+    const int B = T.B, cen = T.cen, team = T.team, nsol = T.nsol, VL = T.VL, GL = T.GL;
+    const Shape& S = T.shape[8 + KIND_RING];
+    const int nl = S.nl, nt = S.nt, K = S.K, a0 = S.a0, c0 = S.c0;
+    const AxisWin wz = T.win[pass_pos(jo, B, cen).M];
+    const int Lz = wz.L, za = wz.ia, dz = wz.ib - wz.ia;
+    const TeamSolve t0 = tm_solve(i, B, cen, team);
+    const bool bwd = t0.bwd;
+    const int dy = (bwd != (t0.role == ROLE_U)) ? -1 : 1;
+    const int lsrc = dy > 0 ? nl - 1 : 0, ldst = nl - 1 - lsrc;   // the line that feeds the next block, the one that takes it
+    const float fs = bwd ? 1.f : -1.f;
+    int y = T.win[t0.Mp].lo + T.win[t0.Mp].ia;            // the block's first line
+    const long long* po = T.soff + t0.Mp;
+    int ri = slot_of_solve(i, nsol, cen, team);
+    const int sh = __ffs(nl) - 1;                         // nl is a power of two
+    const int l = ii & (nl - 1), src = lane + 4 * (l == ldst ? lsrc - ldst : 0);
+    Upd u = *up;
+    bool ok = true;
+#pragma unroll 1
+    for (; i < end && ok; ++i, y += dy * nl, po += dy) {
+        ++u.tag;
+        const float2 kc = dy > 0 ? T.cdn[y + nl] : T.cup[y - 1];
+        const float2 k = make_float2(fs * kc.x, fs * kc.y);
+        const float* sc = A.scale + *po + ii;
+        float2* line = T.V + (y + l) * VL;
+        const float2* gl = T.Gv + (y + dy * nl + l) * GL;
+        float2* zl = T.Zv + (y + l) * GL;
+        const int rn = i + 1 == nsol - 1 ? SLOT_END : (!team && i + 1 == cen ? SLOT_CENTRE : (ri + 1) & (NRING - 1));
+        unsigned char* X = T.X + rn * A.slot_bytes + part_offset(cb, lane);
+        u64* H = T.H + rn * A.hdr_words + cb * 4;
+        int2 ec = make_int2(0, 0), ep = ec;
+#pragma unroll 1
+        for (int tl = 0; (tl < nt || tl == 0) && ok; ++tl) {
+            const int p0 = tl * GT + gi0;
+            const bool fv = !idle && p0 < c0, fv1 = NRS == 2 && p0 + 4 < c0;
+            // operands of this thread's rows, in flight during the product
+            int fe[NRS], fz[NRS], er[NRS], ei[NRS];
+            float4 pre[NRS];
+#pragma unroll
+            for (int j = 0; j < NRS; ++j) {
+                const int gid = a0 + p0 + 4 * j, r = 8 * gid + ii;
+                const int e = r >> sh, x = e / Lz, lz = e - x * Lz;
+                fe[j] = (j ? fv1 : fv) && r < K ? e * RG + rhs0 : -1;
+                fz[j] = fe[j] >= 0 && lz >= za && lz < za + dz ? (x * dz + lz - za) * RG + rhs0 : -1;
+                pre[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                er[j] = ei[j] = 0;
+                if (fe[j] >= 0) {
+                    er[j] = __float_as_int(ptx::ld_nc_f32_here(sc + 16 * gid));
+                    ei[j] = __float_as_int(ptx::ld_nc_f32_here(sc + 16 * gid + 8));
+                }
+                const int o = bwd ? fe[j] : fz[j];
+                if (o >= 0) pre[j] = ptx::ld_cg_f32x4_here((bwd ? line : gl) + o);
+            }
+            if (tl == 0) {
+                if (!(ok = wait_phase(&T.eready, u.xph, T.limit, &T.abort))) break;
+                u.xph ^= 1u;
+                ec = *reinterpret_cast<const int2*>(&T.ecol[rhs0]);
+                ep = *reinterpret_cast<const int2*>(&T.epred[rhs0]);
+            }
+            float R[NRS][4] = {}, I[NRS][4] = {};
+            if (!(ok = read_tile<RG, MT, NRS>(T, u, S, tlane, split, fv, R, I))) break;
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&T.tfree);
+            float4 W[NRS];
+#pragma unroll
+            for (int j = 0; j < NRS; ++j)
+                if (j ? fv1 : fv) W[j] = scale_rows(R[j], I[j], (er[j] >> 23) - 127, (ei[j] >> 23) - 127, ec.x, ec.y);
+            unsigned hw[NRS];
+#pragma unroll
+            for (int j = 0; j < NRS; ++j)
+                if (j ? fv1 : fv) {
+                    if (bwd) W[j] = sub4(pre[j], W[j]);
+                    if (fe[j] < 0) W[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float4 q = cmul2(k, W[j]);
+                    q = make_float4(__shfl_sync(0xffffffffu, q.x, src), __shfl_sync(0xffffffffu, q.y, src),
+                                    __shfl_sync(0xffffffffu, q.z, src), __shfl_sync(0xffffffffu, q.w, src));
+                    if (l != ldst) q = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (!bwd) q = add4(q, pre[j]);
+                    hw[j] = store_parts(X + (size_t)(a0 + p0 + 4 * j) * KGB, q, ep.x, ep.y);
+                }
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < NRS; ++j)
+                if (j ? fv1 : fv) release_header(H + (a0 + p0 + 4 * j) * NB * 4, hw[j], u.tag + 1u);
+#pragma unroll
+            for (int j = 0; j < NRS; ++j) {
+                const int o = bwd ? fz[j] : fe[j];
+                if (o >= 0) *reinterpret_cast<float4*>((bwd ? zl : line) + o) = W[j];
+            }
+        }
+        ri = rn & (NRING - 1);
+    }
+    *up = u;
+    return ok;
+}
+
+// First solve after the run of run_lines or run_blocks that starts with solve i (i itself: none).
+__device__ __forceinline__ int run_end(Sm& T, int jo, int i) {
     const int B = T.B, cen = T.cen, team = T.team, nsol = T.nsol;
     const Shape& S = T.shape[8 + KIND_RING];
-    if (kind_of(i, nsol, cen, team) != KIND_RING || S.nl != 1 || S.nt != 1) return i;
-    // backward up to the last solve; forward up to the front's last solve (two fronts: it feeds the
-    // centre) or the centre, which has to be one line
-    if (tm_solve(i, B, cen, team).bwd) return nsol - 1;
+    if (kind_of(i, nsol, cen, team) != KIND_RING || 8 % S.nl != 0) return i;
+    // backward up to the last solve, which takes one line; forward up to the front's last solve (two
+    // fronts: it feeds the centre) or the centre, which has to have as many lines
+    if (tm_solve(i, B, cen, team).bwd) return S.nl == 1 ? nsol - 1 : nsol - 2;
     if (T.two) return (team ? T.U : cen) - 1;
-    return T.shape[8 + KIND_CENTRE].nl == 1 ? cen : cen - 1;
+    return T.shape[8 + KIND_CENTRE].nl == S.nl ? cen : cen - 1;
 }
 
 // A solve of any shape.
@@ -1508,9 +1624,10 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
             const int last = jo < nvis ? nsol : 0;
 #pragma unroll 1
             for (int i = 0; i < last && ok;) {
-                const int n = lines_end<MT>(S_, jo, i);
+                const int n = run_end(S_, jo, i);
                 if (n > i) {
-                    ok = run_lines<RG, MT>(A, &S_, &u, jo, i, n);
+                    const Shape& R = S_.shape[8 + KIND_RING];
+                    ok = R.nl == 1 && R.nt == 1 ? run_lines<RG, MT>(A, &S_, &u, jo, i, n) : run_blocks<RG, MT>(A, &S_, &u, jo, i, n);
                     i = n;
                 } else {
                     ok = run_general<RG, MT>(A, &S_, &u, jo, i);
@@ -1589,9 +1706,11 @@ bool plan_groups(const helm_ctx* h, int nr, int G, TeamPlan* P) {
     const SolveGeo gt = tm_geo(win[Mt], win[Mt], N, Mt, 0, B, two);
     const int cg = tm_ceil(gt.K / gt.in.nl, 8);
     int C = std::max(1, std::min(h->dclus / (P->G * P->T), gmin));
-    // row groups of a rank; at least TEAM_MIN_GROUPS (below that more ranks only add headers and
-    // polls), then as few ranks as keep that number
-    const int want = std::max(tm_ceil(cg, C), tm_ceil(h->team_min_groups, gt.in.nl));
+    // groups of columns of a rank; its row groups at least team_min_groups with one line (below that
+    // more ranks only add headers and polls), a group of columns with two (the longer rows stream
+    // slower: n = 50, one front, d = 2 with 24 right-hand sides 23.8 -> 22.1 ms), then as few ranks as
+    // keep that number
+    const int want = std::max(tm_ceil(cg, C), std::max(1, h->team_min_groups / gt.in.nl));
     C = std::min(C, tm_ceil(cg, want));
     P->C = C;
     P->MT = gt.in.nl * tm_ceil(cg, C) <= 4 ? 64 : 128;
