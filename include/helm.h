@@ -85,9 +85,10 @@ typedef struct {
                             reports HELM_ETIMEOUT through helm_status           */
     long long wait_cycles; /* bound of every device-side wait of a HELM_DENSE
                             apply, in SM clock cycles; 0 = 4e9 (about 2 s)       */
-    int    dense_clusters; /* HELM_DENSE: clusters of 8 CTAs in the apply launch;
-                            0 = as many as the GPU holds at once (at most 16);
-                            larger values are clamped to that                   */
+    int    dense_clusters; /* HELM_DENSE: bounds the apply launch to that many
+                            times 8 CTAs; 0 = as many as the GPU holds at once
+                            (FP32: clusters of 8, at most 16; the FP16 forms: one
+                            CTA per SM); larger values are clamped to that      */
     int    reserved_;    /* 0                                                     */
 } helm_opts;
 

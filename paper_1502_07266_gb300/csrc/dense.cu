@@ -21,10 +21,10 @@
 // Setup: the quasi-1D problems are factored chunk by chunk (the twisted block
 // LDU of factor.cu into a temporary buffer), k_dense_G solves with the unit
 // columns of R_in^T and keeps the rows of R_out, and k_dense_pack stores G in
-// the apply's tiles: complex FP32 for the SIMT form, FP16 hi + lo (or hi only)
-// with one power-of-two scale per real row for the tensor-core forms.
+// the FP32 apply's tiles.  The tensor-core forms (FP16 hi + lo parts, or hi) pack and
+// apply it in team.cu.
 //
-// Apply: one persistent launch of clusters of 8 CTAs walks the (2B-1)^2 solves
+// FP32 apply: one persistent launch of clusters of 8 CTAs walks the (2B-1)^2 solves
 // of Algorithm 6 over Algorithm 4 in order (dense_sched.h: with two fronts a
 // step carries a lower-front and an upper-front solve on two groups of
 // clusters).  A solve computes Y = G q for up to 64 right-hand sides: cluster c
@@ -35,8 +35,9 @@
 // through a shared-memory ring with bulk copies), the 8 partial products are
 // summed through distributed shared memory, and the owner of each output row
 // applies the step's update (store, subtract, restrict to the output).  Step
-// s+1 starts when every CTA has arrived on a global counter for step s.  All waits are bounded by a clock limit; on expiry the kernel
-// sets the error word, drains its copies, frees its TMEM and returns.
+// s+1 starts when every CTA has arrived on a global counter for step s.  All waits are
+// bounded by a clock limit; on expiry the kernel sets the error word, drains its copies
+// and returns.
 #include "helm_internal.h"
 #include "ptx.cuh"
 
@@ -337,8 +338,8 @@ k_dense_G(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __restric
 // over the next factor block.  The sums run in k_dense_G's order and round as there:
 // the same bits.
 // Setup at n = 95, two fronts, b_aux = 2 (blocks of 9 to 25): 479 -> 173 ms.  What bounds it
-// then is the operator entries' way to memory and back (19.8 GB, 2.9 ms each) and the
-// steps' chain of shared-memory products.
+// then is the steps' chain of dependent shared-memory products; the operator entries' way
+// to memory and back (19.8 GB, 2.9 ms each) is 3 % of it.
 template <int KM>
 __global__ void __launch_bounds__(GW)
 k_dense_G_cols(Geom g, Tables t, const DProb* __restrict__ dp, const GItem* __restrict__ items, int nitems,
@@ -1252,7 +1253,7 @@ __global__ void __launch_bounds__(DT, 1) k_dense(const __grid_constant__ DenseAr
         }
     }
     named_sync_compute();
-    // ---- teardown: let issued copies land, free TMEM, leave with the cluster ----
+    // ---- teardown: let issued copies land, leave with the cluster ----
     if (tid == 0) {
         const int issued = *s_issued;
         int q = consumed % DSTAGES;
@@ -1575,8 +1576,8 @@ int dense_setup(helm_ctx* h, const void* win_host, const void* prob_host, cudaSt
     return HELM_OK;
 }
 
-// Right-hand sides of one apply launch padded to a power of two >= 8 (the MMA
-// width is 4 x that, the gather maps 256 threads onto the columns).
+// Right-hand sides of one apply launch padded to a power of two >= 8 (the gather maps
+// 256 threads onto the columns).
 static int dense_r8(int nr) {
     int r = 8;
     while (r < nr) r <<= 1;

@@ -1,8 +1,9 @@
 // Step schedule of the dense apply (Algorithm 6 over Algorithm 4, one front or
 // Section 4.2's two fronts): which quasi-1D solve a step of the persistent
-// launch carries, and on which clusters.  Plain integer code, shared by the
-// kernel and by the host-side schedule test; included inside dense.cu's
-// anonymous namespace.
+// launch carries, and on which clusters (the FP32 form's; the team apply uses the pass
+// positions and operator slots).  Plain integer code, shared by the kernels and by the
+// host-side schedule test; included inside the anonymous namespace of dense.cu and of
+// team.cu.
 #pragma once
 
 // Position j (0 .. 2B-2) of a block sweep (Algorithm 4 or 6) with centre block

@@ -61,7 +61,6 @@ struct DProb {
     int nkc;            // K-chunks of at most 128 per rank
     int xr;             // extra rows per tile (0..2), stored in complex FP32 after the tile
     long long off;      // byte offset of the operator's tiles
-    long long soff;     // float offset of its per-row scales (FP16 forms)
 };
 
 // A stored operator of the tensor-core forms (team_map.h): the same index sets,

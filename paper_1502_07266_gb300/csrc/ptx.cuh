@@ -1,15 +1,15 @@
-// Inline-PTX wrappers for sm_103a used by the dense apply kernel: mbarriers,
+// Inline-PTX wrappers for sm_103a used by the dense apply kernels: mbarriers,
 // bulk copies, distributed shared memory, and the fifth-generation tensor
 // core (tcgen05: TMEM allocation, MMA issue and commit, TMEM loads).
 //
 // Shared-memory matrix descriptors follow the tcgen05 "matrix descriptor"
 // format: start address, leading-dimension and stride-dimension byte offsets
 // (all >> 4), the fixed version bits 46-48 = 0b001, base offset 0, relative
-// LBO mode, no swizzle.  Operands are K-major and built from 8-row x 16-byte
-// core matrices (8 x 8 FP16 values, 128 contiguous bytes): in this library a
-// tile of R rows x kw K-values stores core matrix (row group g, K group kg) at
-// byte g * SBO + kg * 128 with SBO = (kw / 8) * 128, so LBO (next core matrix
-// along K) is 128 and one K = 16 MMA step advances the start address by 256.
+// LBO mode, no swizzle.  Operands are built from core matrices of 8 rows x 16 bytes
+// (8 x 8 FP16 values, 128 contiguous bytes).  A is K-major: a tile of R rows x kw
+// K-values stores core matrix (row group g, K group kg) at byte g * SBO + kg * 128 with
+// SBO = (kw / 8) * 128, so LBO (next core matrix along K) is 128 and one K = 16 MMA step
+// advances the start address by 256.  B is N-major (umma_idesc_f16_bn).
 #pragma once
 
 #include <stdint.h>
@@ -213,13 +213,5 @@ __device__ __forceinline__ void reg_tie4(float (&v)[4]) {
 // Then reg_tie4: every use of v depends on that statement, so none is scheduled
 // before the wait (volatile statements keep their order).
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// Waits for the warp's outstanding TMEM loads; the registers are tied to the
-// wait so that no use is scheduled before it.
-__device__ __forceinline__ void tmem_wait8(float (&a)[8], float (&b)[8]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]),
-                   "+f"(b[0]), "+f"(b[1]), "+f"(b[2]), "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7])
-                 :: "memory");
-}
 
 }  // namespace ptx
