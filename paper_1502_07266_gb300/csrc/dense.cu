@@ -1512,39 +1512,41 @@ int dense_setup(helm_ctx* h, const void* win_host, const void* prob_host, cudaSt
     const int B = h->g.B;
     const int P = dense_nops(B);
     cudaError_t e;
-    // ---- the apply launch: clusters of 8 CTAs, as many as can be resident (<= 16) ----
+    // ---- the FP32 form's apply launch: clusters of 8 CTAs, as many as can be resident (<= 16) ----
     h->dsmem = dense_smem_bytes(B);
     if (B > DENSE_MAX_B) return HELM_ENOTSUP;
     const bool fp32 = h->opts.precision == HELM_FP32;
+    const void* kfn = dense_kernel_for(h->g.sched);
+    e = ensure_dyn_smem(kfn, h->dsmem);
+    if (e != cudaSuccess) { helm_set_cuda_error(e); return HELM_ECUDA; }
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = HELM_DENSE_CS;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(HELM_DENSE_CS * 16, 1, 1);
+    cfg.blockDim = dim3(DT, 1, 1);
+    cfg.dynamicSmemBytes = h->dsmem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int ncl = 0;
+    e = cudaOccupancyMaxActiveClusters(&ncl, kfn, &cfg);
+    if (e != cudaSuccess) { helm_set_cuda_error(e); return HELM_ECUDA; }
+    if (ncl < 1) return HELM_ENOTSUP;
+    // the tensor-core forms take the tiles of this launch for the rows they keep in more than 16 bits
+    int nclus = std::min(ncl, 16);
+    if (h->opts.dense_clusters > 0) nclus = std::min(nclus, h->opts.dense_clusters);
     if (fp32) {
-        const void* kfn = dense_kernel_for(h->g.sched);
-        e = ensure_dyn_smem(kfn, h->dsmem);
-        if (e != cudaSuccess) { helm_set_cuda_error(e); return HELM_ECUDA; }
-        cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof(cfg));
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = HELM_DENSE_CS;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(HELM_DENSE_CS * 16, 1, 1);
-        cfg.blockDim = dim3(DT, 1, 1);
-        cfg.dynamicSmemBytes = h->dsmem;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int ncl = 0;
-        e = cudaOccupancyMaxActiveClusters(&ncl, kfn, &cfg);
-        if (e != cudaSuccess) { helm_set_cuda_error(e); return HELM_ECUDA; }
-        if (ncl < 1) return HELM_ENOTSUP;
-        h->dclus = std::min(ncl, 16);
-        if (h->opts.dense_clusters > 0) h->dclus = std::min(h->dclus, h->opts.dense_clusters);
+        h->dclus = nclus;
     } else {
         const int rc = team_configure(h);
         if (rc != HELM_OK) return rc;
     }
     std::vector<DProb> dp;
     size_t gbytes = 0, nscale = 0;
-    build_dense_table(h, win, h->dclus, dp, &gbytes);
+    build_dense_table(h, win, nclus, dp, &gbytes);
     if (!fp32) {
         h->tprob_h = new TProb[P];
         team_table(h, dp.data(), h->tprob_h, &gbytes, &nscale);

@@ -70,7 +70,8 @@ struct TProb {
     DRect out[2], in;
     int ng0, ng1;       // row groups of the out rects
     int KP;             // padded input columns
-    int pad_;
+    int halves;         // 2: hi and lo parts are stored, 1: hi parts
+    int xr;             // FP16 form: the last xr of every 64 + xr rows keep their lo parts
     long long off;      // byte offset of the operator's chunks
     long long soff;     // float offset of its per-row scales (16 per group)
 };
@@ -159,6 +160,7 @@ struct helm_ctx {
     TProb* tprob_h;          // and on the host
     void* win_h;             // host copy of the axis windows (AxisWin[B])
     int team_min_groups;     // least row groups of 8 per rank of a team
+    int team_halves;         // most parts an operator stores (TProb::halves)
     size_t dsmem;            // dynamic shared memory of the apply kernel
 };
 
@@ -201,7 +203,7 @@ size_t dense_work_elems(const helm_ctx* h, int nrhs, size_t limit);
 size_t dense_noalloc_elems(const helm_ctx* h, int nrhs);
 void dense_free(helm_ctx* h);
 // Tensor-core forms of the dense apply (team.cu).
-void team_table(const helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t* nscale);
+void team_table(helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t* nscale);
 cudaError_t team_pack(helm_ctx* h, const int* ops, int nops, const float2* Gt, const long long* d_goff,
                       void** d_items, size_t* cap, cudaStream_t st);
 cudaError_t team_unpack(helm_ctx* h, int p, float2* G, cudaStream_t st);

@@ -98,8 +98,8 @@ struct PackItem { int p, gr; };
 
 // One row group (8 complex rows) of operator p, from its complex FP32 rows in Gt
 // (dense.cu's entry order) into the chunks of team_map.h, with one power-of-two
-// scale per real row.
-template <int HALVES>
+// scale per real row.  In the FP16 form an operator with xr > 0 keeps hi parts alone
+// but for the last xr of every 64 + xr rows.
 __global__ void __launch_bounds__(128)
 k_team_pack(const TProb* __restrict__ tp, const PackItem* __restrict__ items, const float2* __restrict__ Gt,
             const long long* __restrict__ goff, unsigned char* __restrict__ G, float* __restrict__ scale, int N) {
@@ -109,7 +109,7 @@ k_team_pack(const TProb* __restrict__ tp, const PackItem* __restrict__ items, co
     const TProb D = tp[I.p];
     const float2* src = Gt + goff[I.p];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ng = D.ng0 + D.ng1, n_in = D.n_in, KP = D.KP;
+    const int ng = D.ng0 + D.ng1, n_in = D.n_in, KP = D.KP, halves = D.halves;
     if (tid < 8) {
         const int q = I.gr >= D.ng0;
         const DRect R = D.out[q];
@@ -149,6 +149,7 @@ k_team_pack(const TProb* __restrict__ tp, const PackItem* __restrict__ items, co
         const int row = e & 7, k8 = e >> 3, c = (8 * k8) / TKC;
         const int kc = min(TKC, KP - c * TKC), kk = 8 * k8 - c * TKC;
         const int o = s_row[row];
+        const bool hi_only = D.xr > 0 && o % (64 + D.xr) < 64;
         __align__(16) __half hi[2][8], lo[2][8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -162,17 +163,17 @@ k_team_pack(const TProb* __restrict__ tp, const PackItem* __restrict__ items, co
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 hi[p][u] = __float2half_rn(v[p]);
-                lo[p][u] = __float2half_rn(v[p] - __half2float(hi[p][u]));
+                lo[p][u] = __float2half_rn(hi_only ? 0.f : v[p] - __half2float(hi[p][u]));
             }
         }
         int bytes;
-        const size_t bh = tm_tile(c, 0, I.gr, ng, KP, HALVES, &bytes);
+        const size_t bh = tm_tile(c, 0, I.gr, ng, KP, halves, &bytes);
         const size_t pos = (size_t)(kk >> 3) * 128 + row * 16;
 #pragma unroll
         for (int p = 0; p < 2; ++p)
             *reinterpret_cast<uint4*>(dst + bh + (size_t)p * kc * 16 + pos) = *reinterpret_cast<const uint4*>(hi[p]);
-        if (HALVES == 2) {
-            const size_t bl = tm_tile(c, 1, I.gr, ng, KP, HALVES, &bytes);
+        if (halves == 2) {
+            const size_t bl = tm_tile(c, 1, I.gr, ng, KP, halves, &bytes);
 #pragma unroll
             for (int p = 0; p < 2; ++p)
                 *reinterpret_cast<uint4*>(dst + bl + (size_t)p * kc * 16 + pos) =
@@ -183,7 +184,6 @@ k_team_pack(const TProb* __restrict__ tp, const PackItem* __restrict__ items, co
 
 // Reads one stored operator back as complex FP32 [n_out][n_in] in dense.cu's
 // entry order (for tests).
-template <int HALVES>
 __global__ void k_team_unpack(TProb D, const unsigned char* __restrict__ G, const float* __restrict__ scale, int N,
                               float2* __restrict__ out) {
     const int ng = D.ng0 + D.ng1;
@@ -206,9 +206,9 @@ __global__ void k_team_unpack(TProb D, const unsigned char* __restrict__ G, cons
         for (int p = 0; p < 2; ++p) {
             int bytes;
             const size_t pos = (size_t)p * kc * 16 + (size_t)(kk >> 3) * 128 + row * 16 + (kk & 7) * 2;
-            float v = __half2float(*reinterpret_cast<const __half*>(G + D.off + tm_tile(c, 0, gr, ng, D.KP, HALVES, &bytes) + pos));
-            if (HALVES == 2)
-                v += __half2float(*reinterpret_cast<const __half*>(G + D.off + tm_tile(c, 1, gr, ng, D.KP, HALVES, &bytes) + pos));
+            float v = __half2float(*reinterpret_cast<const __half*>(G + D.off + tm_tile(c, 0, gr, ng, D.KP, D.halves, &bytes) + pos));
+            if (D.halves == 2)
+                v += __half2float(*reinterpret_cast<const __half*>(G + D.off + tm_tile(c, 1, gr, ng, D.KP, D.halves, &bytes) + pos));
             part[p] = v / scale[D.soff + (long long)gr * 16 + p * 8 + row];
         }
         out[e] = make_float2(part[0], part[1]);
@@ -248,7 +248,7 @@ struct TeamArgs {
     int* err;
     size_t slot_bytes, start_bytes;
     int hdr_words, start_words;
-    int nrhs, T, C, halves;
+    int nrhs, T, C;
     int DZ, Emax, KB;       // KB: input entries a gather pass holds (multiple of TKC)
     int stages, stage_bytes;
     int off_b, off_misc;    // shared memory: the B operand, the rest (the ring starts at 0)
@@ -385,12 +385,13 @@ struct Shape {
     int a0, c0, a1, c1;           // this rank's row groups [a, a + c) of the two out rects
     int ng0, ng, nt, kg0;         // row groups of rect 0 and of the operator, tiles, first own input group
     int kg1, nl, nz, z0;          // end of the own input groups; the in rect's lines, z rows and first row
+    int halves;                   // 2: the operator has lo parts
 };
 __device__ __forceinline__ int kind_of(int i, int nsol, int cen, int upper) {
     return i == 0 ? KIND_START : (i == nsol - 1 ? KIND_END : (!upper && i == cen ? KIND_CENTRE : KIND_RING));
 }
 
-__device__ __noinline__ void make_shapes(Shape* out, const AxisWin* win, int N, int B, int cen, int two, int upper,
+__device__ __noinline__ void make_shapes(Shape* out, const AxisWin* win, const TProb* tp, int N, int B, int cen, int two, int upper,
                                          int M, int rank, int C, int GT, int lane) {
     __syncwarp();
     if (lane < 4) {
@@ -425,6 +426,7 @@ __device__ __noinline__ void make_shapes(Shape* out, const AxisWin* win, int N, 
         s.nl = g.in.nl;
         s.nz = g.in.nz;
         s.z0 = g.in.z0;
+        s.halves = tp[op_index(M, op_slot(t.Mp, t.bwd, B), B)].halves;
         out[lane] = s;
     }
     __syncwarp();
@@ -709,7 +711,7 @@ __device__ __noinline__ bool general_rows(const TeamArgs& A, Sm* T, Upd* pu, int
     const int p0 = tl * GT + gi0, np = S.c0 + S.c1;
     float R[NRS][4] = {}, I[NRS][4] = {};
     Upd u = *pu;
-    const bool ok = read_tile<RG, MT, NRS>(*T, u, S, tlane, A.halves == 2, !idle && p0 < np, R, I);
+    const bool ok = read_tile<RG, MT, NRS>(*T, u, S, tlane, S.halves == 2, !idle && p0 < np, R, I);
     *pu = u;
     if (!ok) return false;
     ptx::tc_fence_before();
@@ -881,7 +883,7 @@ __device__ __noinline__ bool begin_visit(const TeamArgs& A, Sm* Tp, Upd* up, int
     bool ok = cta_sync(T, u, T.limit);                 // everybody is done with the records of the visit before
     *up = u;
     if (tid < 32) {
-        make_shapes(shapes, T.win, T.N, B, cen, T.two, team, M, T.rank, T.C, MT / 16, tid & 31);
+        make_shapes(shapes, T.win, A.tp, T.N, B, cen, T.two, team, M, T.rank, T.C, MT / 16, tid & 31);
         // the entries that pad an input are the last rank's, zero for the whole visit
         const unsigned slots = T.rank == T.C - 1 ? used_slots(nsol, cen, team) : 0u;
 #pragma unroll 1
@@ -918,11 +920,11 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
     const bool idle = RG == 8 && MT == 64 && hh == 1;     // no accumulator columns for this warp
     constexpr int SUBC = acc_slots(RG, MT) * 4 * RG;
     const uint32_t tlane = T.tslot + ((uint32_t)(32 * q4) << 16) + 32 * cb + (gi0 >> 2) * SUBC;
-    const bool split = A.halves == 2;
     const int B = T.B, cen = T.cen, team = T.team, nsol = T.nsol;
     const AxisWin wz = T.win[pass_pos(jo, B, cen).M];
     const int Lz = wz.L, za = wz.ia, dz = wz.ib - wz.ia, E = T.N * Lz;
     const Shape& S = T.shape[8 + KIND_RING];
+    const bool split = S.halves == 2;
     int cg0, cg1;                                         // this rank's groups of 8 columns
     tm_part(E, 1, 1, T.rank, T.C, &cg0, &cg1);
     cg0 += gi0;                                           // this warp's (first) group
@@ -1034,9 +1036,9 @@ __device__ __noinline__ bool run_blocks(const TeamArgs& A, Sm* Tp, Upd* up, int 
     const int gi0 = RG == 8 && MT == 128 ? warp : q4;
     const bool idle = RG == 8 && MT == 64 && hh == 1;
     const uint32_t tlane = T.tslot + ((uint32_t)(32 * q4) << 16) + 32 * cb + (gi0 >> 2) * SUBC;
-    const bool split = A.halves == 2;
     const int B = T.B, cen = T.cen, team = T.team, nsol = T.nsol, VL = T.VL, GL = T.GL;
     const Shape& S = T.shape[8 + KIND_RING];
+    const bool split = S.halves == 2;
     const int nl = S.nl, nt = S.nt, K = S.K, a0 = S.a0, c0 = S.c0;
     const AxisWin wz = T.win[pass_pos(jo, B, cen).M];
     const int Lz = wz.L, za = wz.ia, dz = wz.ib - wz.ia;
@@ -1282,7 +1284,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
         bool ok = true;
         for (int jo = 0; jo < nvis && ok; ++jo) {
             const int M = pass_pos(jo, B, cen).M;
-            make_shapes(shapes, s_win, N, B, cen, two, team, M, rank, C, GT, lane);
+            make_shapes(shapes, s_win, A.tp, N, B, cen, two, team, M, rank, C, GT, lane);
             for (int q = lane; q < B + 2; q += 32) s_off[q] = A.tp[op_index(M, q, B)].off;
             __syncwarp();
 #pragma unroll 1
@@ -1303,13 +1305,13 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                     for (int kc0 = 0; kc0 < KP; kc0 += TKC) {
                         ok = wait_phase(&empty[stage], eph, limit, s_abort);
                         if (!ok) break;
-                        const int kc = min(TKC, KP - kc0), per = 32 * kc * A.halves;      // bytes of a group
+                        const int kc = min(TKC, KP - kc0), per = 32 * kc * S.halves;      // bytes of a group
                         if (lane == 0)
                             ptx::mbar_expect_tx(&full[stage], (uint32_t)((g1 - g0) * per));
                         __syncwarp();
                         if (lane < 2 && cnt > 0)
                             ptx::bulk_g2s(ring + stage * A.stage_bytes + (run ? m0 : 0) * per,
-                                          base + ((size_t)kc0 * ng + (size_t)kc * gr) * A.halves * 32,
+                                          base + ((size_t)kc0 * ng + (size_t)kc * gr) * S.halves * 32,
                                           (uint32_t)(cnt * per), &full[stage]);
                         ++issued;
                         if (++stage == A.stages) { stage = 0; eph ^= 1u; }
@@ -1332,7 +1334,6 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
         // the whole warp runs the loop: uniform operands, one elected lane issues; nothing is called
         // (after a call the compiler takes nothing for uniform), the gather warp makes the records
         const Shape* shapes = s_shape + 4;
-        const uint32_t idesc = ptx::umma_idesc_f16_bn(A.halves == 2 ? 128 : 64, 4 * RG);
         const uint64_t bdesc0 = ptx::umma_desc(ptx::smem_u32(Bbuf), KGB, 128u);
         const uint32_t a_s = ptx::smem_u32(ring);
         int stage = 0, seen = 0;                                  // seen: chunks ahead known to have landed
@@ -1356,6 +1357,8 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                 const int nu = __shfl_sync(0xffffffffu, S.nu, 0), cpa = __shfl_sync(0xffffffffu, S.cpa, 0);
                 const int w = __shfl_sync(0xffffffffu, S.w, 0), NU = SLOTS >> (w >> 1);
                 const int rsh = __shfl_sync(0xffffffffu, S.rsh, 0), per = rsh == 2 ? 1 : w;   // per: accumulators of a chunk or run
+                const int hv = __shfl_sync(0xffffffffu, S.halves, 0);
+                const uint32_t idesc = ptx::umma_idesc_f16_bn(64 * hv, 4 * RG);
                 const bool passes = KP > A.KB;                    // every tile gathers the input anew, in passes
 #pragma unroll 1
                 for (int tl = 0; (tl < nt || tl == 0) && ok; ++tl) {
@@ -1398,7 +1401,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                                 const uint32_t d = tmem + (uint32_t)((us * w + va) * ACOLS);
                                 const uint32_t ahi = a_s + (uint32_t)(stage * A.stage_bytes), sbo = (uint32_t)(kc * 16);
                                 const uint64_t ad = ptx::umma_desc(ahi, 128u, sbo);
-                                chunk_products<RG, NSUB>(d, ad, 8 * A.halves * sbo / 16, bd, idesc, ca > 0, rsh, kc);
+                                chunk_products<RG, NSUB>(d, ad, 8 * hv * sbo / 16, bd, idesc, ca > 0, rsh, kc);
                                 bd += TKC / 16 * 2 * KGB / 16;
                                 ptx::umma_commit_warp(&empty[stage]);
                                 if (++stage == A.stages) { stage = 0; fph ^= 1u; }
@@ -1442,7 +1445,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                 mph ^= 1u;
                 fresh = true;
             }
-            make_shapes(shapes, s_win, N, B, cen, two, team, pass_pos(jo, B, cen).M, rank, C, GT, lane);
+            make_shapes(shapes, s_win, A.tp, N, B, cen, two, team, pass_pos(jo, B, cen).M, rank, C, GT, lane);
             ri = 0;
 #pragma unroll 1
             for (int i = 0; i < nsol && ok; ++i) {
@@ -1676,7 +1679,7 @@ bool plan_groups(const helm_ctx* h, int nr, int G, TeamPlan* P) {
     const int N = h->g.N, B = h->g.B, cen = h->g.cen;
     const bool two = h->g.sched == HELM_TWO_FRONT;
     const AxisWin* win = static_cast<const AxisWin*>(h->win_h);
-    const int halves = h->opts.precision == HELM_FP16 ? 1 : 2;
+    const int halves = h->team_halves;
     P->T = two ? 2 : 1;
     // one block of 8 right-hand sides, or groups of 16: the operator is streamed once per group
     P->RG = nr <= 8 ? 8 : 16;
@@ -1768,9 +1771,10 @@ const void* team_kernel(int RG, int MT) {
 }  // namespace
 
 // Operator table of the tensor-core forms; fills the byte and scale counts.
-void team_table(const helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t* nscale) {
+void team_table(helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t* nscale) {
     const int N = h->g.N, P = dense_nops(h->g.B);
-    const int halves = h->opts.precision == HELM_FP16 ? 1 : 2;
+    const bool fp16 = h->opts.precision == HELM_FP16;
+    h->team_halves = fp16 ? 1 : 2;
     size_t off = 0, soff = 0;
     for (int p = 0; p < P; ++p) {
         TProb t;
@@ -1787,7 +1791,10 @@ void team_table(const helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, s
             t.ng0 = tm_ceil(D.out[0].nl * D.out[0].nz * N, 8);
             t.ng1 = D.nrect > 1 ? tm_ceil(D.out[1].nl * D.out[1].nz * N, 8) : 0;
             t.KP = tm_kp(D.n_in);
-            off += tm_bytes(t.ng0 + t.ng1, t.KP, halves);
+            t.xr = fp16 ? D.xr : 0;
+            t.halves = fp16 && D.xr == 0 ? 1 : 2;
+            h->team_halves = std::max(h->team_halves, t.halves);
+            off += tm_bytes(t.ng0 + t.ng1, t.KP, t.halves);
             soff += (size_t)(t.ng0 + t.ng1) * 16;
         }
         tp[p] = t;
@@ -1815,10 +1822,7 @@ cudaError_t team_pack(helm_ctx* h, const int* ops, int nops, const float2* Gt, c
     const PackItem* di = static_cast<const PackItem*>(*d_items);
     e = cudaMemcpyAsync(*d_items, items.data(), items.size() * sizeof(PackItem), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
-    if (h->opts.precision == HELM_FP16)
-        k_team_pack<1><<<(unsigned)items.size(), 128, 0, st>>>(h->tprob, di, Gt, d_goff, h->dG, h->dscale, h->g.N);
-    else
-        k_team_pack<2><<<(unsigned)items.size(), 128, 0, st>>>(h->tprob, di, Gt, d_goff, h->dG, h->dscale, h->g.N);
+    k_team_pack<<<(unsigned)items.size(), 128, 0, st>>>(h->tprob, di, Gt, d_goff, h->dG, h->dscale, h->g.N);
     h->launches++;
     e = cudaGetLastError();
     // the item list above must outlive its copy
@@ -1827,10 +1831,7 @@ cudaError_t team_pack(helm_ctx* h, const int* ops, int nops, const float2* Gt, c
 }
 
 cudaError_t team_unpack(helm_ctx* h, int p, float2* G, cudaStream_t st) {
-    if (h->opts.precision == HELM_FP16)
-        k_team_unpack<1><<<512, 256, 0, st>>>(h->tprob_h[p], h->dG, h->dscale, h->g.N, G);
-    else
-        k_team_unpack<2><<<512, 256, 0, st>>>(h->tprob_h[p], h->dG, h->dscale, h->g.N, G);
+    k_team_unpack<<<512, 256, 0, st>>>(h->tprob_h[p], h->dG, h->dscale, h->g.N, G);
     h->launches++;
     return cudaGetLastError();
 }
@@ -1855,6 +1856,7 @@ int team_configure(helm_ctx* h) {
     h->dclus = nsm;
     if (h->opts.dense_clusters > 0) h->dclus = std::min(h->dclus, HELM_DENSE_CS * h->opts.dense_clusters);
     h->team_min_groups = 3;
+    h->team_halves = 2;                  // until the operators are known
     if (h->dclus < (h->g.sched == HELM_TWO_FRONT ? 2 : 1)) return HELM_ENOTSUP;
     TeamPlan P;
     return team_plan(h, 1, &P, (size_t)-1) && team_plan(h, 64, &P, (size_t)-1) ? HELM_OK : HELM_ENOTSUP;
@@ -1901,7 +1903,6 @@ cudaError_t launch_team_apply(helm_ctx* h, const float2* r, float2* z, int nrhs,
         A.nrhs = nr;
         A.T = P.T;
         A.C = P.C;
-        A.halves = h->opts.precision == HELM_FP16 ? 1 : 2;
         A.DZ = P.DZ;
         A.Emax = P.Emax;
         A.KB = P.KB;
