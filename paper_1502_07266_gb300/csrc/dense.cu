@@ -1545,11 +1545,12 @@ int dense_setup(helm_ctx* h, const void* win_host, const void* prob_host, cudaSt
         if (rc != HELM_OK) return rc;
     }
     std::vector<DProb> dp;
+    std::vector<int> lo;
     size_t gbytes = 0, nscale = 0;
     build_dense_table(h, win, nclus, dp, &gbytes);
     if (!fp32) {
         h->tprob_h = new TProb[P];
-        team_table(h, dp.data(), h->tprob_h, &gbytes, &nscale);
+        team_table(h, dp.data(), h->tprob_h, &gbytes, &nscale, &lo);
     }
     h->dprob_h = new DProb[P];
     memcpy(h->dprob_h, dp.data(), sizeof(DProb) * P);
@@ -1562,6 +1563,10 @@ int dense_setup(helm_ctx* h, const void* win_host, const void* prob_host, cudaSt
     }
     DTRY(cudaMalloc(&h->dG, gbytes));
     h->dG_bytes = gbytes;
+    if (!lo.empty()) {
+        DTRY(cudaMalloc(&h->dlo, lo.size() * sizeof(int)));
+        DTRY(cudaMemcpyAsync(h->dlo, lo.data(), lo.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+    }
     if (nscale) {
         DTRY(cudaMalloc(&h->dscale, nscale * sizeof(float)));
         h->dscale_elems = nscale;
@@ -1670,7 +1675,7 @@ int dense_rebuild(helm_ctx* h, int Ma, int Mb, int Pa, int Pb, cudaStream_t st) 
 }
 
 void dense_free(helm_ctx* h) {
-    void* ptrs[] = {h->dprob, h->tprob, h->dG, h->dscale, h->dV};
+    void* ptrs[] = {h->dprob, h->tprob, h->dG, h->dscale, h->dlo, h->dV};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete[] h->dprob_h;
@@ -1681,6 +1686,7 @@ void dense_free(helm_ctx* h) {
     h->dprob_h = nullptr;
     h->dG = nullptr;
     h->dscale = nullptr;
+    h->dlo = nullptr;
     h->dV = nullptr;
 }
 

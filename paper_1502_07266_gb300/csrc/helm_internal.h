@@ -5,6 +5,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <vector>
+
 #include "../../include/helm.h"
 
 #define HELM_KMAX 64          // largest quasi-1D block (window lines x layers)
@@ -72,6 +74,7 @@ struct TProb {
     int KP;             // padded input columns
     int halves;         // 2: hi and lo parts are stored, 1: hi parts
     int xr;             // FP16 form: the last xr of every 64 + xr rows keep their lo parts
+    int nlo, lob;       // row groups with such rows, and the place of their table (TProb::nlo > 0: halves is 2)
     long long off;      // byte offset of the operator's chunks
     long long soff;     // float offset of its per-row scales (16 per group)
 };
@@ -158,6 +161,7 @@ struct helm_ctx {
                              // tensor-core forms: CTAs it may use
     TProb* tprob;            // tensor-core forms: the operator table on the device
     TProb* tprob_h;          // and on the host
+    int* dlo;                // FP16 form: a unit of zeros, then per row group the number of its lo parts or -1
     void* win_h;             // host copy of the axis windows (AxisWin[B])
     int team_min_groups;     // least row groups of 8 per rank of a team
     int team_halves;         // most parts an operator stores (TProb::halves)
@@ -203,7 +207,7 @@ size_t dense_work_elems(const helm_ctx* h, int nrhs, size_t limit);
 size_t dense_noalloc_elems(const helm_ctx* h, int nrhs);
 void dense_free(helm_ctx* h);
 // Tensor-core forms of the dense apply (team.cu).
-void team_table(helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t* nscale);
+void team_table(helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t* nscale, std::vector<int>* lo);
 cudaError_t team_pack(helm_ctx* h, const int* ops, int nops, const float2* Gt, const long long* d_goff,
                       void** d_items, size_t* cap, cudaStream_t st);
 cudaError_t team_unpack(helm_ctx* h, int p, float2* G, cudaStream_t st);

@@ -12,7 +12,7 @@
 // cross CTAs, and groups never wait for one another.
 //
 // What bounds it: the latency of one solve, i.e. epilogue -> publish -> gather ->
-// product, 31.6 thousand times in a row at n = 127.  Measured on GB300 (cycles at 2.07
+// product, 33 thousand times in a row at n = 127.  Measured on GB300 (cycles at 2.07
 // GHz): bulk copies from L2 land 550 cycles after their issue and stream at about
 // 60 B/clk on every SM at once; distributed shared memory moves 20 B/clk, so an
 // all-gather of 27 kB takes 1.9 k cycles there, and of 55 kB 3.1 k; publishing
@@ -30,10 +30,11 @@
 // formed: it comes from the largest entry of the solve before and of the slab
 // right-hand side on the next line (a table made in the boundary phase), with
 // room for a growth by 2^7; entries down to 2^-10 of that maximum keep both parts in
-// full, smaller ones an absolute error of 2^-33 of it.  A rank whose entries do
+// full, smaller ones an absolute error of 2^-33 of it.  So an input that shrinks by 2^k
+// against what its scale comes from loses k bits more.  A rank whose entries do
 // not fit (they grew more) scales them by their own maximum and says so in the
 // header of the 8 entries; a gather that finds unequal scales brings them to the
-// smallest in shared memory before the product.
+// smallest in shared memory before the product (in FP16: the same absolute error).
 //
 // Headers carry the solve's number and are released at GPU scope after the parts; the
 // gathering warp reads them until they are all there, fences (acquire, and a proxy
@@ -99,10 +100,11 @@ struct PackItem { int p, gr; };
 // One row group (8 complex rows) of operator p, from its complex FP32 rows in Gt
 // (dense.cu's entry order) into the chunks of team_map.h, with one power-of-two
 // scale per real row.  In the FP16 form an operator with xr > 0 keeps hi parts alone
-// but for the last xr of every 64 + xr rows.
+// but for the last xr of every 64 + xr rows, whose groups have lo parts (lo: which).
 __global__ void __launch_bounds__(128)
 k_team_pack(const TProb* __restrict__ tp, const PackItem* __restrict__ items, const float2* __restrict__ Gt,
-            const long long* __restrict__ goff, unsigned char* __restrict__ G, float* __restrict__ scale, int N) {
+            const long long* __restrict__ goff, unsigned char* __restrict__ G, float* __restrict__ scale, const int* __restrict__ lo,
+            int N) {
     __shared__ int s_row[8];
     __shared__ float s_sc[16];
     const PackItem I = items[blockIdx.x];
@@ -150,7 +152,7 @@ k_team_pack(const TProb* __restrict__ tp, const PackItem* __restrict__ items, co
         const int kc = min(TKC, KP - c * TKC), kk = 8 * k8 - c * TKC;
         const int o = s_row[row];
         const bool hi_only = D.xr > 0 && o % (64 + D.xr) < 64;
-        __align__(16) __half hi[2][8], lo[2][8];
+        __align__(16) __half hi[2][8], lw[2][8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int k = 8 * k8 + u;
@@ -163,29 +165,30 @@ k_team_pack(const TProb* __restrict__ tp, const PackItem* __restrict__ items, co
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 hi[p][u] = __float2half_rn(v[p]);
-                lo[p][u] = __float2half_rn(hi_only ? 0.f : v[p] - __half2float(hi[p][u]));
+                lw[p][u] = __float2half_rn(hi_only ? 0.f : v[p] - __half2float(hi[p][u]));
             }
         }
         int bytes;
-        const size_t bh = tm_tile(c, 0, I.gr, ng, KP, halves, &bytes);
+        const int idx = D.nlo ? lo[D.lob + I.gr] : 0;
+        const size_t bh = D.nlo ? tm_unit(c, I.gr, ng + D.nlo, KP) : tm_tile(c, 0, I.gr, ng, KP, halves, &bytes);
         const size_t pos = (size_t)(kk >> 3) * 128 + row * 16;
 #pragma unroll
         for (int p = 0; p < 2; ++p)
             *reinterpret_cast<uint4*>(dst + bh + (size_t)p * kc * 16 + pos) = *reinterpret_cast<const uint4*>(hi[p]);
-        if (halves == 2) {
-            const size_t bl = tm_tile(c, 1, I.gr, ng, KP, halves, &bytes);
+        if (halves == 2 && idx >= 0) {
+            const size_t bl = D.nlo ? tm_unit(c, ng + idx, ng + D.nlo, KP) : tm_tile(c, 1, I.gr, ng, KP, halves, &bytes);
 #pragma unroll
             for (int p = 0; p < 2; ++p)
                 *reinterpret_cast<uint4*>(dst + bl + (size_t)p * kc * 16 + pos) =
-                    *reinterpret_cast<const uint4*>(lo[p]);
+                    *reinterpret_cast<const uint4*>(lw[p]);
         }
     }
 }
 
 // Reads one stored operator back as complex FP32 [n_out][n_in] in dense.cu's
 // entry order (for tests).
-__global__ void k_team_unpack(TProb D, const unsigned char* __restrict__ G, const float* __restrict__ scale, int N,
-                              float2* __restrict__ out) {
+__global__ void k_team_unpack(TProb D, const unsigned char* __restrict__ G, const float* __restrict__ scale,
+                              const int* __restrict__ lo, int N, float2* __restrict__ out) {
     const int ng = D.ng0 + D.ng1;
     const int n0 = D.out[0].nl * D.out[0].nz * N;
     const long long total = (long long)D.n_out * D.n_in;
@@ -202,13 +205,15 @@ __global__ void k_team_unpack(TProb D, const unsigned char* __restrict__ G, cons
         const int per = D.in.nz * D.in.nl, xi = j / per, r = j - xi * per;
         const int k = (xi * D.in.nz + r % D.in.nz) * D.in.nl + r / D.in.nz;
         const int c = k / TKC, kc = min(TKC, D.KP - c * TKC), kk = k - c * TKC;
+        int bytes;
+        const int idx = D.nlo ? lo[D.lob + gr] : 0;
+        const size_t bh = D.nlo ? tm_unit(c, gr, ng + D.nlo, D.KP) : tm_tile(c, 0, gr, ng, D.KP, D.halves, &bytes);
+        const size_t bl = D.nlo ? tm_unit(c, ng + max(idx, 0), ng + D.nlo, D.KP) : tm_tile(c, 1, gr, ng, D.KP, D.halves, &bytes);
         float part[2];
         for (int p = 0; p < 2; ++p) {
-            int bytes;
             const size_t pos = (size_t)p * kc * 16 + (size_t)(kk >> 3) * 128 + row * 16 + (kk & 7) * 2;
-            float v = __half2float(*reinterpret_cast<const __half*>(G + D.off + tm_tile(c, 0, gr, ng, D.KP, D.halves, &bytes) + pos));
-            if (D.halves == 2)
-                v += __half2float(*reinterpret_cast<const __half*>(G + D.off + tm_tile(c, 1, gr, ng, D.KP, D.halves, &bytes) + pos));
+            float v = __half2float(*reinterpret_cast<const __half*>(G + D.off + bh + pos));
+            if (D.halves == 2 && idx >= 0) v += __half2float(*reinterpret_cast<const __half*>(G + D.off + bl + pos));
             part[p] = v / scale[D.soff + (long long)gr * 16 + p * 8 + row];
         }
         out[e] = make_float2(part[0], part[1]);
@@ -233,6 +238,7 @@ struct TeamArgs {
     const TProb* tp;
     const unsigned char* G;
     const float* scale;
+    const int* lo;          // FP16 form: a chunk's unit of zeros, then the numbers of the groups' lo parts (-1: none)
     const float2* c_dn;
     const float2* c_up;
     const float2* rin;
@@ -385,7 +391,7 @@ struct Shape {
     int a0, c0, a1, c1;           // this rank's row groups [a, a + c) of the two out rects
     int ng0, ng, nt, kg0;         // row groups of rect 0 and of the operator, tiles, first own input group
     int kg1, nl, nz, z0;          // end of the own input groups; the in rect's lines, z rows and first row
-    int halves;                   // 2: the operator has lo parts
+    int halves, nlo, lob;         // 2: the operator has lo parts; nlo > 0: of that many groups (table at lob)
 };
 __device__ __forceinline__ int kind_of(int i, int nsol, int cen, int upper) {
     return i == 0 ? KIND_START : (i == nsol - 1 ? KIND_END : (!upper && i == cen ? KIND_CENTRE : KIND_RING));
@@ -426,7 +432,10 @@ __device__ __noinline__ void make_shapes(Shape* out, const AxisWin* win, const T
         s.nl = g.in.nl;
         s.nz = g.in.nz;
         s.z0 = g.in.z0;
-        s.halves = tp[op_index(M, op_slot(t.Mp, t.bwd, B), B)].halves;
+        const TProb& D = tp[op_index(M, op_slot(t.Mp, t.bwd, B), B)];
+        s.halves = D.halves;
+        s.nlo = D.nlo;
+        s.lob = D.lob;
         out[lane] = s;
     }
     __syncwarp();
@@ -1280,6 +1289,7 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
         // ------------------------------------------- operator stream -> ring
         Shape* shapes = s_shape;
         int stage = 0, issued = 0;
+        uint32_t zeros = 0;                  // stages where this lane's part is zero
         uint32_t eph = 1;                    // the first round finds every stage free
         bool ok = true;
         for (int jo = 0; jo < nvis && ok; ++jo) {
@@ -1301,18 +1311,44 @@ __global__ void __launch_bounds__(TT, 1) k_team(const __grid_constant__ TeamArgs
                     const int run = lane & 1;
                     const int cnt = run ? g1 - g0 - m0 : m0;
                     const int gr = run ? S.ng0 + S.a1 + max(0, g0 - c0) : S.a0 + g0;
+                    // lo parts of some groups only: every group's parts for themselves (lane & 1: lo), zeros where there
+                    // are none (not again into a stage whose place holds them: copying them each time made an
+                    // apply of such operators 20 % longer)
+                    const int mg = lane >> 1, nlo = S.nlo;
+                    int unit = 0;
+                    bool some = false;
+                    if (nlo && mg < g1 - g0) {
+                        const int q = mg < m0 ? S.a0 + g0 + mg : S.ng0 + S.a1 + max(0, g0 - c0) + mg - m0;
+                        unit = run ? __ldg(A.lo + S.lob + q) : q;
+                        some = unit >= 0;
+                        if (run) unit += ng;
+                    }
 #pragma unroll 1
                     for (int kc0 = 0; kc0 < KP; kc0 += TKC) {
                         ok = wait_phase(&empty[stage], eph, limit, s_abort);
                         if (!ok) break;
                         const int kc = min(TKC, KP - kc0), per = 32 * kc * S.halves;      // bytes of a group
-                        if (lane == 0)
-                            ptx::mbar_expect_tx(&full[stage], (uint32_t)((g1 - g0) * per));
-                        __syncwarp();
-                        if (lane < 2 && cnt > 0)
-                            ptx::bulk_g2s(ring + stage * A.stage_bytes + (run ? m0 : 0) * per,
-                                          base + ((size_t)kc0 * ng + (size_t)kc * gr) * S.halves * 32,
-                                          (uint32_t)(cnt * per), &full[stage]);
+                        if (nlo) {
+                            const bool mine = mg < g1 - g0, none = mine && run && !some && kc == TKC;
+                            const bool go = mine && !(none && (zeros >> stage & 1u));
+                            const unsigned n = __popc(__ballot_sync(0xffffffffu, go));
+                            if (lane == 0) ptx::mbar_expect_tx(&full[stage], n * 32u * (uint32_t)kc);
+                            __syncwarp();
+                            if (go)
+                                ptx::bulk_g2s(ring + stage * A.stage_bytes + mg * per + run * 32 * kc,
+                                              some ? base + tm_unit(kc0 / TKC, unit, ng + nlo, KP)
+                                                   : reinterpret_cast<const unsigned char*>(A.lo),
+                                              (uint32_t)(32 * kc), &full[stage]);
+                            zeros = none ? zeros | 1u << stage : zeros & ~(1u << stage);
+                        } else {
+                            if (lane == 0) ptx::mbar_expect_tx(&full[stage], (uint32_t)((g1 - g0) * per));
+                            __syncwarp();
+                            if (lane < 2 && cnt > 0)
+                                ptx::bulk_g2s(ring + stage * A.stage_bytes + (run ? m0 : 0) * per,
+                                              base + ((size_t)kc0 * ng + (size_t)kc * gr) * S.halves * 32,
+                                              (uint32_t)(cnt * per), &full[stage]);
+                            zeros &= ~(1u << stage);
+                        }
                         ++issued;
                         if (++stage == A.stages) { stage = 0; eph ^= 1u; }
                     }
@@ -1770,8 +1806,10 @@ const void* team_kernel(int RG, int MT) {
 
 }  // namespace
 
-// Operator table of the tensor-core forms; fills the byte and scale counts.
-void team_table(helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t* nscale) {
+// Operator table of the tensor-core forms; fills the byte and scale counts.  lo, where an
+// operator has lo parts of some groups only: a unit of zeros, which stands for the others'
+// parts, then of each such shape, per row group, the number of its lo parts or -1.
+void team_table(helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t* nscale, std::vector<int>* lo) {
     const int N = h->g.N, P = dense_nops(h->g.B);
     const bool fp16 = h->opts.precision == HELM_FP16;
     h->team_halves = fp16 ? 1 : 2;
@@ -1793,8 +1831,34 @@ void team_table(helm_ctx* h, const DProb* dp, TProb* tp, size_t* gbytes, size_t*
             t.KP = tm_kp(D.n_in);
             t.xr = fp16 ? D.xr : 0;
             t.halves = fp16 && D.xr == 0 ? 1 : 2;
+            if (t.xr > 0) {
+                // a shape seen before has its table already
+                int q = 0;
+                while (q < p && !(tp[q].nlo > 0 && tp[q].xr == t.xr && tp[q].n_out == t.n_out && tp[q].ng0 == t.ng0 &&
+                                  tp[q].out[0].nl == t.out[0].nl && tp[q].out[0].nz == t.out[0].nz &&
+                                  tp[q].out[1].nl == t.out[1].nl && tp[q].out[1].nz == t.out[1].nz))
+                    ++q;
+                if (q < p) {
+                    t.nlo = tp[q].nlo;
+                    t.lob = tp[q].lob;
+                } else {
+                    if (lo->empty()) lo->assign(TKC * 32 / sizeof(int), 0);
+                    t.lob = (int)lo->size();
+                    for (int g = 0; g < t.ng0 + t.ng1; ++g) {
+                        const int r = g >= t.ng0, n0 = t.out[0].nl * t.out[0].nz * N;
+                        const DRect& R = t.out[r];
+                        bool some = false;
+                        for (int u = 0; u < 8; ++u) {
+                            const int i = 8 * (g - (r ? t.ng0 : 0)) + u, l = i % R.nl, tt = i / R.nl, zr = tt % R.nz, x = tt / R.nz;
+                            const int o = (r ? n0 : 0) + x + N * (zr + R.nz * l);
+                            some = some || (x < N && o % (64 + t.xr) >= 64);
+                        }
+                        lo->push_back(some ? t.nlo++ : -1);
+                    }
+                }
+            }
             h->team_halves = std::max(h->team_halves, t.halves);
-            off += tm_bytes(t.ng0 + t.ng1, t.KP, t.halves);
+            off += t.nlo > 0 ? (size_t)(t.ng0 + t.ng1 + t.nlo) * t.KP * 32 : tm_bytes(t.ng0 + t.ng1, t.KP, t.halves);
             soff += (size_t)(t.ng0 + t.ng1) * 16;
         }
         tp[p] = t;
@@ -1822,7 +1886,7 @@ cudaError_t team_pack(helm_ctx* h, const int* ops, int nops, const float2* Gt, c
     const PackItem* di = static_cast<const PackItem*>(*d_items);
     e = cudaMemcpyAsync(*d_items, items.data(), items.size() * sizeof(PackItem), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
-    k_team_pack<<<(unsigned)items.size(), 128, 0, st>>>(h->tprob, di, Gt, d_goff, h->dG, h->dscale, h->g.N);
+    k_team_pack<<<(unsigned)items.size(), 128, 0, st>>>(h->tprob, di, Gt, d_goff, h->dG, h->dscale, h->dlo, h->g.N);
     h->launches++;
     e = cudaGetLastError();
     // the item list above must outlive its copy
@@ -1831,7 +1895,7 @@ cudaError_t team_pack(helm_ctx* h, const int* ops, int nops, const float2* Gt, c
 }
 
 cudaError_t team_unpack(helm_ctx* h, int p, float2* G, cudaStream_t st) {
-    k_team_unpack<<<512, 256, 0, st>>>(h->tprob_h[p], h->dG, h->dscale, h->g.N, G);
+    k_team_unpack<<<512, 256, 0, st>>>(h->tprob_h[p], h->dG, h->dscale, h->dlo, h->g.N, G);
     h->launches++;
     return cudaGetLastError();
 }
@@ -1883,6 +1947,7 @@ cudaError_t launch_team_apply(helm_ctx* h, const float2* r, float2* z, int nrhs,
         A.tp = h->tprob;
         A.G = h->dG;
         A.scale = h->dscale;
+        A.lo = h->dlo;
         A.c_dn = h->t.c_dn;
         A.c_up = h->t.c_up;
         A.rin = r + (size_t)r0 * n3;

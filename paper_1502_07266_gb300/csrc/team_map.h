@@ -126,6 +126,12 @@ __host__ __device__ __forceinline__ size_t tm_tile(int c, int h, int gr, int ng,
     *bytes = 2 * kc * 16;
     return ((size_t)c * TKC * halves * ng + (size_t)kc * (gr * halves + h)) * 32;
 }
+// The same where only some groups have lo parts (nlo of them): a chunk holds units of
+// (16 real rows) x kc, the hi parts of all ng groups, then the lo parts there are.
+__host__ __device__ __forceinline__ size_t tm_unit(int c, int unit, int units, int KP) {
+    const int kc = KP - c * TKC < TKC ? KP - c * TKC : TKC;
+    return ((size_t)c * TKC * units + (size_t)kc * unit) * 32;
+}
 __host__ __device__ __forceinline__ size_t tm_bytes(int ng, int KP, int halves) {
     return (size_t)ng * KP * halves * 32;
 }

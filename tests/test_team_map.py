@@ -93,6 +93,22 @@ int main() {
                 for (int v : hit) once = once && v == 1;
                 printf("T %d %d %d %d\n", halves, K, ng, once);
             }
+    // the same where some groups have lo parts: units
+    for (int K : {16, 64, 65, 417})
+        for (int units : {2, 45}) {
+            const int KP = tm_kp(K);
+            std::vector<int> hit((size_t)units * KP * 32, 0);
+            bool once = true;
+            for (int c = 0; c * TKC < KP; ++c)
+                for (int u = 0; u < units; ++u) {
+                    const int kc = KP - c * TKC < TKC ? KP - c * TKC : TKC;
+                    const size_t o = tm_unit(c, u, units, KP);
+                    for (int q = 0; q < 32 * kc; ++q)
+                        if (o + q < hit.size()) ++hit[o + q]; else once = false;
+                }
+            for (int v : hit) once = once && v == 1;
+            printf("T 0 %d %d %d\n", K, units, once);
+        }
     return 0;
 }
 '''
