@@ -20,8 +20,8 @@
 // the exchange goes through L2.  One apply, split FP16, two fronts: n = 127 with 64
 // right-hand sides 314 ms (K split over clusters of 8, partial sums through
 // distributed shared memory and one step counter for all CTAs: 16.7 k cycles a
-// solve) -> 181 ms; n = 63 with one 57.8 -> 40.3 ms; one front, n = 50 with 33,
-// FP16 operators 103 -> 58 ms.
+// solve) -> 191 ms; n = 63 with one 57.8 -> 40.3 ms; one front, n = 50 with 33,
+// FP16 operators 104 -> 62 ms.
 //
 // Exchange.  q is published as FP16 hi + lo parts in the layout of the tensor
 // core's B operand (N-major core matrices), so a gather is a plain bulk copy into
@@ -375,15 +375,20 @@ __device__ __forceinline__ void chunk_products(uint32_t d, uint64_t ad, uint32_t
 // the code larger than the instruction caches: 258 kB and 5 to 8 cycles per
 // instruction).
 //
-// An accumulator takes a run of products: a quarter of the input's, an eighth beyond 32
-// products, rounded down to 1, 2 or a multiple of 4 so that runs and chunks end together.  The products signal a few accumulators at a
-// time, a unit: those of a chunk, or two, or one where there are at most four.  Before the
-// teams every input went into eight partial sums; error of a split FP16 apply against 64
-// bits then, with four accumulators of whole chunks, and now: n = 33, two fronts, b_aux 1 (6
-// products, so two accumulators) 6.4e-6, 8.0e-6, 4.6e-6; n = 50, one front, b_aux 3 (16)
-// 8.9e-6, 8.5e-6, 8.5e-6; the same with d = 2 (39) 8.1e-6, 6.7e-6, 4.3e-6.  Reading an accumulator costs a warp 150 cycles or more: runs of
-// an eighth for all give n = 50 6.0e-6 in 64.8 ms instead of 60.2, n = 63 with one right-hand
-// side 43.2 ms instead of 40.6.
+// An accumulator takes a run of products, rounded down to 1, 2 or a multiple of 4 so that
+// runs and chunks end together: a quarter of the input's, 2 up to 14 products, and at most
+// 8 or an eighth.  With FP16 operators 2 up to 16 products and 4 up to 32: what they lose in
+// the chain is the only difference from eight partial sums, and adds up over the solves (n
+// = 111, two fronts, b_aux 1, 16 products: runs of 4 moved results by 1.3e-5, locally 3.3e-4;
+// runs of 2 by 1.5e-6).  The products signal a few accumulators at a time, a unit: those of a
+// chunk, or two, or one where there are at most four.  Before the teams every input went
+// into eight partial sums; error of a split FP16 apply against 64 bits then, with an
+// accumulator for every chunk or more, and now: n = 33, two fronts, b_aux 1 (6 products)
+// 6.4e-6, 8.0e-6, 4.6e-6; n = 31, one front, b_aux 4 (14) 4.3e-6, 4.5e-6, 3.9e-6; n = 50, one
+// front, b_aux 3 (16) 8.9e-6, 8.5e-6, 8.5e-6; the same with d = 2 (39) 8.1e-6, 6.7e-6, 6.4e-6.
+// Reading an accumulator costs a warp 150 cycles or more: runs of an eighth for all give n
+// = 50 6.0e-6 in 64.8 ms instead of 60.2 and n = 63 with one right-hand side 43.2 ms instead of
+// 40.6; at 27 products runs of 8 gave n = 127 9.4e-6 in 188.5 ms, those of 4 5.4e-6 in 190.6.
 enum { KIND_START = 0, KIND_RING = 1, KIND_CENTRE = 2, KIND_END = 3 };
 struct Shape {
     int K, KP;                    // input entries, padded to a multiple of 16
@@ -421,7 +426,11 @@ __device__ __noinline__ void make_shapes(Shape* out, const AxisWin* win, const T
         s.ng0 = tm_ceil(g.n0, 8);
         s.ng = s.ng0 + tm_ceil(g.n1, 8);
         s.nt = tm_ceil(s.c0 + s.c1, GT);
-        const int n16 = s.KP / 16, nch = tm_ceil(s.KP, TKC), run = tm_ceil(n16, n16 <= 32 ? 4 : 8);
+        const int n16 = s.KP / 16, nch = tm_ceil(s.KP, TKC), q = tm_ceil(n16, 4);
+        const TProb& D = tp[op_index(M, op_slot(t.Mp, t.bwd, B), B)];
+        const bool fp16 = D.halves == 1 || D.nlo > 0;
+        const int run = n16 <= (fp16 ? 16 : 14) ? min(q, 2)
+                                                : (fp16 && n16 <= 32 ? 4 : min(q, max(8, tm_ceil(n16, 8))));
         s.rsh = run >= 4 ? 2 : (run > 1 ? 1 : 0);
         s.cpa = max(1, run / 4);
         const int na = run >= 4 ? tm_ceil(nch, s.cpa) : tm_ceil(n16, 1 << s.rsh);
@@ -432,7 +441,6 @@ __device__ __noinline__ void make_shapes(Shape* out, const AxisWin* win, const T
         s.nl = g.in.nl;
         s.nz = g.in.nz;
         s.z0 = g.in.z0;
-        const TProb& D = tp[op_index(M, op_slot(t.Mp, t.bwd, B), B)];
         s.halves = D.halves;
         s.nlo = D.nlo;
         s.lob = D.lob;
@@ -1032,7 +1040,7 @@ __device__ __noinline__ bool run_lines(const TeamArgs& A, Sm* Tp, Upd* up, int j
 // publishes the groups whose rows it holds, each tile while the next is multiplied.
 // Against run_general (couplings through L2, a barrier of the CTA, index divisions
 // after the product) one apply: two lines, n = 50, one
-// front with 24 right-hand sides 31.0 -> 22.1 ms (the K split over clusters 25.3), n = 30, two
+// front with 24 right-hand sides 31.0 -> 21.4 ms (the K split over clusters 25.3), n = 30, two
 // fronts with 9 6.7 -> 4.5 (5.4), n = 17 with two 1.90 -> 1.44 (1.71)
 template <int RG, int MT>
 __device__ __noinline__ bool run_blocks(const TeamArgs& A, Sm* Tp, Upd* up, int jo, int i, int end) {
