@@ -20,7 +20,7 @@
 // the exchange goes through L2.  One apply, split FP16, two fronts: n = 127 with 64
 // right-hand sides 314 ms (K split over clusters of 8, partial sums through
 // distributed shared memory and one step counter for all CTAs: 16.7 k cycles a
-// solve) -> 191 ms; n = 63 with one 57.8 -> 40.3 ms; one front, n = 50 with 33,
+// solve) -> 191 ms; n = 63 with one 57.8 -> 41.5 ms; one front, n = 50 with 33,
 // FP16 operators 104 -> 62 ms.
 //
 // Exchange.  q is published as FP16 hi + lo parts in the layout of the tensor
